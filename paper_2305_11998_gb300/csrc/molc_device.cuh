@@ -1,0 +1,77 @@
+// Device helpers shared by the CUDA sources of libmolc.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "molc_internal.h"
+
+namespace molc {
+
+// Not (x >= 0 and finite), decided on the bits (integer pipe; the FP64 pipe is narrow): +0, -0 and the positive
+// finite numbers pass.
+__device__ __forceinline__ bool bad_input(double x) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  return !(u < 0x7FF0000000000000ull || u == 0x8000000000000000ull);
+}
+
+// FP32 -> FP64 by integer operations (the FP64 conversion pipe is narrow on this GPU): exponent rebiased by
+// 1023 - 127 and mantissa shifted into place, exact for normal numbers.  Zeros and subnormals (|x| < 2^-126)
+// map to a value of the same sign and magnitude below 2^-126; the FP32 sweep works in units where max B is
+// ~2^100, so that is below 1e-68 of max B.
+__device__ __forceinline__ double f32_to_f64(float x) {
+  const unsigned u = __float_as_uint(x);
+  const unsigned hi = (u & 0x80000000u) | (((u >> 3) & 0x0fffffffu) + 0x38000000u);
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+
+// Exact FP32 -> FP64 for every finite x: the integer route for normal numbers, the conversion instruction for
+// zeros and subnormals.
+__device__ __forceinline__ double f32_to_f64_exact(float x) {
+  return (__float_as_uint(x) & 0x7f800000u) ? f32_to_f64(x) : (double)x;
+}
+
+// What an FP32 sweep adds to the segment update: nothing, the face reductions of Eq. 16 (MOLC_FACES), or the
+// per-ray balance check (MOLC_BALANCE).
+enum SweepExtra { kSweepPlain = 0, kSweepFaces = 1, kSweepBalance = 2 };
+
+// Per-ray balance (MOLC_BALANCE): R = I_in - I_out + sum_s tau_s (d_s - psibar_s), which is the integral of the
+// transport equation along the characteristic, I_in - I_out + sum_s (Q_s - kappa~_s Ibar_s) l_s / sin zeta, in the
+// deviation variables (Q - kappa~ Ibar = kappa~ (d - psibar)).  Segment by segment it reads
+// I_in,s - I_out,s + tau_s (d_s - psibar_s) = 0, and the crossings add I_out,s - I_in,s+1 = 0 (the steps of B the
+// deviation form takes there); S is the sum of the magnitudes of all these terms in the variables the sweep
+// rounds (|I_in,s|, |I_out,s| and their deviations |psi_in,s|, |psi_out,s| from the cell's B, tau_s |B_s + d_s| =
+// |Q_s| l_s / sin zeta, tau_s |B_s + psibar_s| = kappa~_s |Ibar_s| l_s / sin zeta, the B steps), so that |R| / S
+// is a few units of the working precision's rounding when the arithmetic is consistent.  The largest |R| / S goes
+// into *word by an integer atomicMax (non-negative doubles order like their bits).
+// Rays whose terms sum to less than kBalanceFloor of max(B, boundary) (word[1], in the units of R and S after the
+// factor `units`) carry no radiation at the working precision and are left out.
+constexpr double kBalanceFloor = 1e-30;
+__device__ __forceinline__ void ray_balance_max(unsigned long long *word, double R, double S, double units) {
+  const double floor = kBalanceFloor * __longlong_as_double((long long)word[1]) * units;
+  if (!(S > floor) || !(S > 0.0)) return;
+  atomicMax(word, (unsigned long long)__double_as_longlong(fabs(R) / S));
+}
+
+
+// Eddington factors of one (cell, group) from the moments just assembled (Eq. 7 with the cell averages of
+// Eq. 15): f = N / (c E), 0 where E = 0.  The same operations as closure_cells, so molc_sweep_closure and
+// molc_sweep + molc_closure give the same bits.
+__device__ __forceinline__ void eddington_factors(const SweepArgs &a, int64_t idx, double E, double nxx, double nxy,
+                                                  double nyy) {
+  const double inv = E > 0 ? 1.0 / (a.c * E) : 0.0;
+  a.fxx[idx] = nxx * inv;
+  a.fxy[idx] = nxy * inv;
+  a.fyy[idx] = nyy * inv;
+}
+
+// The FP64 sweep's cell entry; 1/(c dt kappa~) rounds like the quotient it replaces.
+__device__ __forceinline__ Cell64 cell64(double kappa, double B, double Bref, double inv_cdt) {
+  Cell64 c;
+  c.kt = kappa + inv_cdt;
+  c.r = inv_cdt / c.kt;
+  c.B = B;
+  c.dB = (Bref - B) * c.r;
+  return c;
+}
+
+}  // namespace molc

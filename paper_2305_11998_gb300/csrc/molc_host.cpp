@@ -94,12 +94,15 @@ struct molc_plan {
   double *d_seg_len = nullptr, *d_seg_afrac = nullptr;
   PairDev *d_pairs = nullptr;
   PolarDev *d_polar = nullptr;
+  PolarFix *d_polar_fix = nullptr;
+  int *d_track_order = nullptr;
   double *d_geo = nullptr;
   int64_t *d_dir_seg_off = nullptr;
   int *d_status = nullptr;
   float4 *d_cdat = nullptr;
   float *d_cdB = nullptr;
   double *d_acc = nullptr;
+  Cell64 *d_cell64 = nullptr;
   int2 *d_items32 = nullptr;
   int64_t n_items32 = 0;
   int64_t *d_cell_off = nullptr;
@@ -362,12 +365,44 @@ void free_device(molc_plan *p) {
   void *ptrs[] = {p->d_tracks, p->d_seg32, p->d_seg_cell, p->d_seg_len, p->d_seg_afrac, p->d_pairs, p->d_polar,
                   p->d_geo, p->d_dir_seg_off, p->d_status, p->d_cdat, p->d_cdB, p->d_acc, p->d_items32,
                   p->d_cell_off, p->d_gent, p->d_boff, p->d_block_order, p->d_seg_face, p->d_facc,
-                  p->d_munit, p->d_mmulti, p->d_mscratch, p->d_balance};
+                  p->d_munit, p->d_mmulti, p->d_mscratch, p->d_balance, p->d_polar_fix, p->d_cell64, p->d_track_order};
   for (void *q : ptrs)
     if (q) cudaFree(q);
   for (void *q : p->tdev)
     if (q) cudaFree(q);
   p->tdev.clear();
+}
+
+// Mantissa (64 bits, normalised) and exponent of a positive normal double: x = M 2^(e - 63).
+unsigned long long mantissa64(double x, int &e) {
+  const double m = std::frexp(x, &e);   // [1/2, 1)
+  --e;
+  return (unsigned long long)std::ldexp(m, 53) << 11;
+}
+
+// The FP64 sweep's constants of one polar cosine, by integer arithmetic from 1/sin zeta (the same on every host).
+PolarFix polar_fixed(const PolarDev &pl) {
+  using u128 = unsigned __int128;
+  constexpr unsigned long long kLog2e = 0xb8aa3b295c17f0bcull;   // log2 e in units of 2^-63
+  PolarFix f{};
+  int e;
+  f.Mi = mantissa64(pl.inv_sinz, e);
+  f.ei = (short)e;
+  auto normalised = [](u128 x, int e, short &eo) {   // x 2^(e - 63) with x >= 2^63
+    while (x >> 64) {
+      x = (x + 1) >> 1;
+      ++e;
+    }
+    eo = (short)e;
+    return (unsigned long long)x;
+  };
+  f.Mz = normalised(((u128)f.Mi * kLog2e + ((u128)1 << 62)) >> 63, f.ei, f.ez);
+  // 2^127 / Mi in (2^63, 2^64]: sin zeta = 2^(-ei) 2^63 / Mi
+  f.Ms = normalised((((u128)1 << 127) + f.Mi / 2) / f.Mi, -f.ei - 1, f.es);
+  f.w = pl.w;
+  f.ws = pl.w * pl.sinz;
+  f.wss = pl.w * pl.sinz * pl.sinz;
+  return f;
 }
 
 bool finite_pos(double x) { return std::isfinite(x) && x > 0; }
@@ -457,7 +492,7 @@ molc_status autotune(molc_plan *p, double *best_ms_out) {
     e = cudaMemset(I, 0, state_bytes_fp32(p));
     if (e == cudaSuccess) e = cudaMemcpy(a.Bref, a.B, cg * sizeof(double), cudaMemcpyDeviceToDevice);
     if (e == cudaSuccess) e = launch_set_scale(p->view, MOLC_FP32, a.B, const_cast<double *>(a.scale), nullptr);
-    if (e == cudaSuccess) e = launch_prep(p->view, MOLC_FP32, a, nullptr);
+    if (e == cudaSuccess) e = launch_prep(p->view, a, nullptr);
     auto timed = [&](int d, int n, float &ms) {
       PlanView v = p->view;
       v.sweep_depth = d;
@@ -1262,6 +1297,16 @@ molc_status molc_create(const molc_grid *grid, const molc_quadrature *quad, cons
     *out = p;
     return MOLC_OK;
   }
+  std::vector<PolarFix> polar_fix;
+  for (const PolarDev &pl : p->polar) polar_fix.push_back(polar_fixed(pl));
+  // FP64 sweep: tracks longest first (a counting sort that keeps the order among equals)
+  int longest = 0;
+  for (const TrackDev &t : td) longest = std::max(longest, t.nseg);
+  std::vector<int64_t> first((size_t)longest + 2, 0);
+  for (const TrackDev &t : td) ++first[(size_t)(longest - t.nseg) + 1];
+  for (size_t k = 1; k < first.size(); ++k) first[k] += first[k - 1];
+  std::vector<int> track_order((size_t)T);
+  for (int64_t k = 0; k < T; ++k) track_order[(size_t)first[(size_t)(longest - td[k].nseg)]++] = (int)k;
   // ---- upload
   molc_status st = MOLC_OK;
   size_t &tot = p->device_bytes;
@@ -1274,6 +1319,8 @@ molc_status molc_create(const molc_grid *grid, const molc_quadrature *quad, cons
   UP(d_seg_afrac, p->seg_afrac.data(), (size_t)S, "segment areas")
   UP(d_pairs, p->pairs.data(), p->pairs.size(), "pairs")
   UP(d_polar, p->polar.data(), p->polar.size(), "polar")
+  UP(d_polar_fix, polar_fix.data(), polar_fix.size(), "polar")
+  UP(d_track_order, track_order.data(), (size_t)T, "track order")
   UP(d_geo, geo.data(), geo.size(), "geometric moments")
   UP(d_dir_seg_off, p->dir_seg_off.data(), p->dir_seg_off.size(), "direction offsets")
   UP(d_status, (const int *)nullptr, 1, "status")
@@ -1291,6 +1338,7 @@ molc_status molc_create(const molc_grid *grid, const molc_quadrature *quad, cons
   UP(d_cdat, (const float4 *)nullptr, (size_t)nch32 * gc32 * ncell, "cell table")
   UP(d_cdB, (const float *)nullptr, (size_t)nch32 * gc32 * ncell, "cell table")
   UP(d_acc, (const double *)nullptr, p->acc_elems, "accumulators")
+  UP(d_cell64, (const Cell64 *)nullptr, (size_t)ncell * p->G, "FP64 cell entries")
   UP(d_items32, items.data(), items.size(), "items")
 #undef UP
   if (st == MOLC_OK) {
@@ -1310,6 +1358,8 @@ molc_status molc_create(const molc_grid *grid, const molc_quadrature *quad, cons
   v.seg_afrac = p->d_seg_afrac;
   v.pairs = p->d_pairs;
   v.polar = p->d_polar;
+  v.polar_fix = p->d_polar_fix;
+  v.track_order = p->d_track_order;
   v.geo = p->d_geo;
   v.dir_seg_off = p->d_dir_seg_off;
   v.status = p->d_status;
@@ -1602,6 +1652,7 @@ static molc_status sweep_step(molc_plan *p, molc_precision prec, const double *k
   a.cdat = p->d_cdat;
   a.cdB = p->d_cdB;
   a.acc = p->d_acc;
+  a.cell64 = p->d_cell64;
   a.items = p->d_items32;
   a.n_items = p->n_items32;
   a.fxx = fxx;
@@ -1617,10 +1668,7 @@ static molc_status sweep_step(molc_plan *p, molc_precision prec, const double *k
     if (e == cudaSuccess) e = launch_balance_scale(p->view, B, bnd, st);
     if (e != cudaSuccess) return cuda_fail(e, who, "balance check set-up");
   }
-  if (prec == MOLC_FP64) {   // the FP32 path gathers its moments and has no accumulators
-    e = cudaMemsetAsync(p->d_acc, 0, (size_t)p->G * p->view.ncell * kOutputs * sizeof(double), st);
-    if (e != cudaSuccess) return cuda_fail(e, who, "clear accumulators");
-  } else {
+  if (prec == MOLC_FP32) {
     e = launch_update_scale(p->view, B, bnd, header_of(p, prec, I), st);
     if (e != cudaSuccess) return cuda_fail(e, who, "scale");
   }
@@ -1634,13 +1682,13 @@ static molc_status sweep_step(molc_plan *p, molc_precision prec, const double *k
     return MOLC_OK;
   }
   if (timed) cudaEventRecord(ev[0], st);
-  e = launch_prep(p->view, prec, a, st);
+  e = prec == MOLC_FP64 ? launch_prep_fp64(p->view, a, st) : launch_prep(p->view, a, st);
   if (e != cudaSuccess) return cuda_fail(e, who, "prep");
   if (timed) cudaEventRecord(ev[1], st);
   e = prec == MOLC_FP64 ? launch_sweep_fp64(p->view, a, st) : launch_sweep_fp32(p->view, a, st);
   if (e != cudaSuccess) return cuda_fail(e, who, "sweep kernel");
   if (timed) cudaEventRecord(ev[2], st);
-  e = launch_finalize(p->view, prec, a, st);
+  e = prec == MOLC_FP64 ? launch_finalize_fp64(p->view, a, st) : launch_moments_fp32(p->view, a, st);
   if (e != cudaSuccess) return cuda_fail(e, who, "finalize");
   if (timed) {
     cudaEventRecord(ev[3], st);
@@ -1709,8 +1757,8 @@ molc_status molc_sweep_static_scratch(molc_plan *p, molc_precision prec, const d
     if (e == cudaSuccess) e = tile_step(p, a, tv, st, nullptr);
     return e == cudaSuccess ? MOLC_OK : cuda_fail(e, "sweep_static_scratch: tiled sweep");
   }
-  // workspace carved from the static array: FP64, the accumulators [cell][6][G] (must start at zero, cleared
-  // below on every call); FP32, the cell tables [chunk][cell][gc] (fully written by prep_kernel)
+  // workspace carved from the static array: FP64, the accumulators [cell][6][G] (cleared by the prep kernel of
+  // every call); FP32, the cell tables [chunk][cell][gc] (fully written by prep_kernel)
   const Layout L = layout_for(p->view, prec);
   const size_t rows = (size_t)L.n_chunks * L.gc * p->view.ncell;
   auto up256 = [](size_t b) { return (b + 255) / 256 * 256; };
@@ -1742,6 +1790,9 @@ molc_status molc_sweep_static_scratch(molc_plan *p, molc_precision prec, const d
   a.scale = header_of(p, prec, I);
   a.out = *out;
   a.acc = prec == MOLC_FP64 ? (double *)b : nullptr;
+  // the FP64 cell entries where they fit behind the accumulators; else the sweep forms them from the inputs
+  if (prec == MOLC_FP64 && acc_bytes + rows * sizeof(Cell64) <= kStaticScratchBytes)
+    a.cell64 = (Cell64 *)(b + acc_bytes);
   a.cdat = prec == MOLC_FP32 ? (float4 *)b : nullptr;
   a.cdB = prec == MOLC_FP32 ? (float *)(b + cdat_bytes) : nullptr;
   a.items = p->d_items32;
@@ -1756,18 +1807,15 @@ molc_status molc_sweep_static_scratch(molc_plan *p, molc_precision prec, const d
     if (e == cudaSuccess) e = launch_balance_scale(p->view, B, bnd, st);
     if (e != cudaSuccess) return cuda_fail(e, "sweep_static_scratch: balance check set-up");
   }
-  if (prec == MOLC_FP64) {
-    e = cudaMemsetAsync(a.acc, 0, rows * kOutputs * sizeof(double), st);
-    if (e != cudaSuccess) return cuda_fail(e, "sweep_static_scratch: clear accumulators");
-  } else {
+  if (prec == MOLC_FP32) {
     e = launch_update_scale(p->view, B, bnd, header_of(p, prec, I), st);
     if (e != cudaSuccess) return cuda_fail(e, "sweep_static_scratch: scale");
   }
-  e = launch_prep(p->view, prec, a, st);
+  e = prec == MOLC_FP64 ? launch_prep_fp64(p->view, a, st) : launch_prep(p->view, a, st);
   if (e != cudaSuccess) return cuda_fail(e, "sweep_static_scratch: prep");
   e = prec == MOLC_FP64 ? launch_sweep_fp64(p->view, a, st) : launch_sweep_fp32(p->view, a, st);
   if (e != cudaSuccess) return cuda_fail(e, "sweep_static_scratch: sweep kernel");
-  e = launch_finalize(p->view, prec, a, st);
+  e = prec == MOLC_FP64 ? launch_finalize_fp64(p->view, a, st) : launch_moments_fp32(p->view, a, st);
   if (e != cudaSuccess) return cuda_fail(e, "sweep_static_scratch: finalize");
   return MOLC_OK;
 }

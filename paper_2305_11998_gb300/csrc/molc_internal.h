@@ -47,6 +47,20 @@ struct PolarDev {       // per (pair, polar cosine)
   int dir_plus, dir_minus;  // quadrature indices of the two directions
 };
 
+// Per (pair, polar cosine), for the FP64 sweep's fixed-point arithmetic: normalised 64-bit mantissas M 2^(e - 63) of
+// log2 e / sin zeta, 1 / sin zeta and its reciprocal; the polar folds' weights omega, omega sin zeta and
+// omega sin^2 zeta.
+struct alignas(16) PolarFix {
+  unsigned long long Mz, Mi, Ms;
+  short ez, ei, es, pad;
+  double w, ws, wss, pad2;
+};
+
+// Per (cell, group), FP64 sweep: kappa~, 1/(c dt kappa~), B, (B_ref - B)/(c dt kappa~).
+struct alignas(32) Cell64 {
+  double kt, r, B, dB;
+};
+
 // Everything a kernel needs, by value.
 struct PlanView {
   int nx, ny, ncell, G, n_pairs, n_polar;
@@ -58,6 +72,8 @@ struct PlanView {
   const double *seg_afrac;      // A / V (area fraction of the cell, after renormalisation)
   const PairDev *pairs;
   const PolarDev *polar;        // [pair][p]
+  const PolarFix *polar_fix;    // [pair][p], FP64 path
+  const int *track_order;       // FP64 path: tracks, longest first
   const double *geo;            // [4][cell]: sum_m omega sum_{C(i,m)} a times 1, Ox^2, OxOy, Oy^2
   const int64_t *dir_seg_off;   // canonical segment offset of each direction
   int *status;
@@ -146,6 +162,7 @@ struct SweepArgs {
   float4 *cdat;       // FP32: [chunk][cell][gc] {kappa~, 1/(c dt kappa~), B_hi, B_lo}
   float *cdB;         // FP32: [chunk][cell][gc] (B_ref - B) / (c dt kappa~)
   double *acc;        // FP64 path: [cell][6][G] FP64 accumulators
+  Cell64 *cell64;     // FP64 path: [cell][G] cell entries, or null (the sweep then forms them from the inputs)
   const int2 *items;  // FP32: one per thread, {track, sense | g_local << 1 | chunk << 16}; chunk-major,
                       // longest track first, then sense, then group
   int64_t n_items;
@@ -162,10 +179,14 @@ struct BatchInst {
 };
 
 // Kernel launchers (molc_kernels.cu).  Return cudaSuccess or the launch error.
-cudaError_t launch_prep(const PlanView &v, molc_precision prec, const SweepArgs &a, cudaStream_t st);
+cudaError_t launch_prep(const PlanView &v, const SweepArgs &a, cudaStream_t st);
 cudaError_t launch_sweep_fp64(const PlanView &v, const SweepArgs &a, cudaStream_t st);
 cudaError_t launch_sweep_fp32(const PlanView &v, const SweepArgs &a, cudaStream_t st);
-cudaError_t launch_finalize(const PlanView &v, molc_precision prec, const SweepArgs &a, cudaStream_t st);
+cudaError_t launch_moments_fp32(const PlanView &v, const SweepArgs &a, cudaStream_t st);
+// FP64 path (molc_fp64.cu): input checks, cell entries and cleared accumulators; the sweep is launch_sweep_fp64; the
+// assembly of the moments (and factors) from the accumulators.
+cudaError_t launch_prep_fp64(const PlanView &v, const SweepArgs &a, cudaStream_t st);
+cudaError_t launch_finalize_fp64(const PlanView &v, const SweepArgs &a, cudaStream_t st);
 cudaError_t launch_closure(const PlanView &v, const molc_moments &m, double c, double *fxx, double *fxy,
                            double *fyy, double *f_grey, cudaStream_t st);
 cudaError_t launch_face_moments(const PlanView &v, molc_precision prec, const double *scale, double c,

@@ -19,6 +19,7 @@
 #include <cstdint>
 #include <mutex>
 
+#include "molc_device.cuh"
 #include "molc_internal.h"
 
 namespace molc {
@@ -26,29 +27,6 @@ namespace molc {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-
-// Not (x >= 0 and finite), decided on the bits (integer pipe; the FP64 pipe is narrow): +0, -0 and the positive
-// finite numbers pass.
-__device__ __forceinline__ bool bad_input(double x) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  return !(u < 0x7FF0000000000000ull || u == 0x8000000000000000ull);
-}
-
-// FP32 -> FP64 by integer operations (the FP64 conversion pipe is narrow on this GPU): exponent rebiased by
-// 1023 - 127 and mantissa shifted into place, exact for normal numbers.  Zeros and subnormals (|x| < 2^-126)
-// map to a value of the same sign and magnitude below 2^-126; the FP32 sweep works in units where max B is
-// ~2^100, so that is below 1e-68 of max B.
-__device__ __forceinline__ double f32_to_f64(float x) {
-  const unsigned u = __float_as_uint(x);
-  const unsigned hi = (u & 0x80000000u) | (((u >> 3) & 0x0fffffffu) + 0x38000000u);
-  return __hiloint2double((int)hi, (int)(u << 29));
-}
-
-// Exact FP32 -> FP64 for every finite x: the integer route for normal numbers, the conversion instruction for
-// zeros and subnormals.
-__device__ __forceinline__ double f32_to_f64_exact(float x) {
-  return (__float_as_uint(x) & 0x7f800000u) ? f32_to_f64(x) : (double)x;
-}
 
 // Track holding row r of the intensity layout (rows are (track, sense, step); a track owns 2 nseg rows).
 __device__ __forceinline__ int64_t find_track(const TrackDev *tr, int64_t T, int64_t row) {
@@ -64,7 +42,7 @@ __device__ __forceinline__ int64_t find_track(const TrackDev *tr, int64_t T, int
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// prep: input checks; FP32 path also tabulates per (chunk, cell, group) {kappa~, 1/(c dt kappa~), B_hi, B_lo}
+// prep (FP32): input checks, and per (chunk, cell, group) {kappa~, 1/(c dt kappa~), B_hi, B_lo}
 // with B = B_hi + B_lo split so that B differences between neighbouring cells keep ~48 bits.
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kPrepCells = 32;   // cells per tile of prep_kernel
@@ -72,7 +50,7 @@ constexpr int kPrepCells = 32;   // cells per tile of prep_kernel
 // Tiles of kPrepCells cells x the groups of one chunk: [g][cell] inputs are read along cells, the
 // [chunk][cell][gc] tables are staged in shared memory and written out contiguously.  A block takes tiles
 // tile0, tile0 + tstride, ...; check_bnd: this block also checks the boundary values.
-__device__ __forceinline__ void prep_tiles(const PlanView &v, const SweepArgs &a, const Layout &L, int fp32,
+__device__ __forceinline__ void prep_tiles(const PlanView &v, const SweepArgs &a, const Layout &L,
                                            int chunk, int tile0, int tstride, bool check_bnd) {
   __shared__ float4 t4[kPrepCells * 32];
   __shared__ float t1[kPrepCells * 32];
@@ -92,148 +70,46 @@ __device__ __forceinline__ void prep_tiles(const PlanView &v, const SweepArgs &a
       const int64_t idx = (int64_t)(g0 + gl) * v.ncell + c0 + c;
       const double kap = a.kappa[idx], B = a.B[idx];
       bad |= bad_input(kap) | bad_input(B);
-      if (fp32) {
-        // FP64 only where a difference or a split needs it (the FP64 pipe is narrow): kappa~ and
-        // 1/(c dt kappa~) are rounded to FP32 anyway and are formed in FP32
-        const float kt = (float)(kap + a.inv_cdt);
-        const float r = __fdiv_rn(inv_cdt_f, kt);
-        const double Bs = B * sc;
-        // !(Bs < kScaledMax) on the bits: signed order is value order for non-negative doubles and -0
-        range |= __double_as_longlong(Bs) >= __double_as_longlong(kScaledMax);
-        const float bhi = (float)Bs;
-        const float blo = (float)(Bs - f32_to_f64_exact(bhi));
-        t4[c * gcount + gl] = make_float4(kt, r, bhi, blo);
-        t1[c * gcount + gl] = (float)((a.Bref[idx] - B) * sc) * r;
-      }
+      // FP64 only where a difference or a split needs it (the FP64 pipe is narrow): kappa~ and
+      // 1/(c dt kappa~) are rounded to FP32 anyway and are formed in FP32
+      const float kt = (float)(kap + a.inv_cdt);
+      const float r = __fdiv_rn(inv_cdt_f, kt);
+      const double Bs = B * sc;
+      // !(Bs < kScaledMax) on the bits: signed order is value order for non-negative doubles and -0
+      range |= __double_as_longlong(Bs) >= __double_as_longlong(kScaledMax);
+      const float bhi = (float)Bs;
+      const float blo = (float)(Bs - f32_to_f64_exact(bhi));
+      t4[c * gcount + gl] = make_float4(kt, r, bhi, blo);
+      t1[c * gcount + gl] = (float)((a.Bref[idx] - B) * sc) * r;
     }
-    if (fp32) {
-      __syncthreads();
-      // [chunk][cell][gc]: the chunk's stride is gc also in a partial last chunk (as the sweep reads it)
-      const int64_t o = (int64_t)g0 * v.ncell + (int64_t)c0 * L.gc;
-      for (int k = threadIdx.x; k < nc * gcount; k += blockDim.x) {
-        const int c = k / gcount, gl = k - c * gcount;
-        a.cdat[o + (int64_t)c * L.gc + gl] = t4[k];
-        a.cdB[o + (int64_t)c * L.gc + gl] = t1[k];
-      }
-      __syncthreads();
+    __syncthreads();
+    // [chunk][cell][gc]: the chunk's stride is gc also in a partial last chunk (as the sweep reads it)
+    const int64_t o = (int64_t)g0 * v.ncell + (int64_t)c0 * L.gc;
+    for (int k = threadIdx.x; k < nc * gcount; k += blockDim.x) {
+      const int c = k / gcount, gl = k - c * gcount;
+      a.cdat[o + (int64_t)c * L.gc + gl] = t4[k];
+      a.cdB[o + (int64_t)c * L.gc + gl] = t1[k];
     }
+    __syncthreads();
   }
   if (check_bnd)
     for (int i = threadIdx.x; i < 4 * v.G; i += blockDim.x) {
       bad |= bad_input(a.bnd[i]);
-      range |= fp32 && !(a.bnd[i] * sc < kScaledMax);
+      range |= !(a.bnd[i] * sc < kScaledMax);
     }
   if (bad) atomicOr(v.status, kStatusNonfinite);
   if (range && !bad) atomicOr(v.status, kStatusRange);
 }
 
-__global__ void __launch_bounds__(128) prep_kernel(PlanView v, SweepArgs a, Layout L, int fp32) {
-  prep_tiles(v, a, L, fp32, blockIdx.y, blockIdx.x, gridDim.x, blockIdx.x == 0 && blockIdx.y == 0);
+__global__ void __launch_bounds__(128) prep_kernel(PlanView v, SweepArgs a, Layout L) {
+  prep_tiles(v, a, L, blockIdx.y, blockIdx.x, gridDim.x, blockIdx.x == 0 && blockIdx.y == 0);
 }
 
 // Batched (FP32): block j prepares tile map[j].z of chunk map[j].y of instance map[j].x.
 __global__ void __launch_bounds__(128) prep_batch_kernel(const BatchInst *inst, const int4 *map) {
   const int4 m = map[blockIdx.x];
   const BatchInst &b = inst[m.x];
-  prep_tiles(b.v, b.a, b.L, 1, m.y, m.z, 1 << 30, m.w != 0);
-}
-
-// ---------------------------------------------------------------------------------------------------------
-// FP64 plain sweep: one thread per (track, sense, group, polar cosine), all arithmetic in FP64, one FP64
-// atomic per output and update into the [cell][6][G] accumulators.
-// Per-ray balance (MOLC_BALANCE): R = I_in - I_out + sum_s tau_s (d_s - psibar_s), which is the integral of the
-// transport equation along the characteristic, I_in - I_out + sum_s (Q_s - kappa~_s Ibar_s) l_s / sin zeta, in the
-// deviation variables (Q - kappa~ Ibar = kappa~ (d - psibar)).  Segment by segment it reads
-// I_in,s - I_out,s + tau_s (d_s - psibar_s) = 0, and the crossings add I_out,s - I_in,s+1 = 0 (the steps of B the
-// deviation form takes there); S is the sum of the magnitudes of all these terms in the variables the sweep
-// rounds (|I_in,s|, |I_out,s| and their deviations |psi_in,s|, |psi_out,s| from the cell's B, tau_s |B_s + d_s| =
-// |Q_s| l_s / sin zeta, tau_s |B_s + psibar_s| = kappa~_s |Ibar_s| l_s / sin zeta, the B steps), so that |R| / S
-// is a few units of the working precision's rounding when the arithmetic is consistent.  The largest |R| / S goes
-// into *word by an integer atomicMax (non-negative doubles order like their bits).
-// Rays whose terms sum to less than kBalanceFloor of max(B, boundary) (word[1], in the units of R and S after the
-// factor `units`) carry no radiation at the working precision and are left out.
-constexpr double kBalanceFloor = 1e-30;
-__device__ __forceinline__ void ray_balance_max(unsigned long long *word, double R, double S, double units) {
-  const double floor = kBalanceFloor * __longlong_as_double((long long)word[1]) * units;
-  if (!(S > floor) || !(S > 0.0)) return;
-  atomicMax(word, (unsigned long long)__double_as_longlong(fabs(R) / S));
-}
-
-// ---------------------------------------------------------------------------------------------------------
-template <bool BAL>   // BAL: with the per-ray balance check (MOLC_BALANCE)
-__global__ void __launch_bounds__(128) sweep_fp64_kernel(PlanView v, SweepArgs a) {
-  const int NP = v.n_polar, Q = v.G * NP;
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= v.n_tracks * 2 * Q) return;
-  const int q = (int)(idx % Q);
-  const int64_t rest = idx / Q;
-  const int sense = (int)(rest & 1);
-  const int64_t t = rest >> 1;
-  const int g = q / NP, p = q - g * NP;
-  const TrackDev tr = v.tracks[t];
-  const PolarDev pd = v.polar[tr.pair * NP + p];
-  const PairDev pr = v.pairs[tr.pair];
-  const double sg = sense ? -1.0 : 1.0;
-  const double Ox = sg * pd.sinz * pr.c, Oy = sg * pd.sinz * pr.s;
-  const double inv_cdt = 1.0 / (a.c * a.dt);
-  const double *kap = a.kappa + (int64_t)g * v.ncell;
-  const double *Bg = a.B + (int64_t)g * v.ncell;
-  const double *Bref = a.Bref + (int64_t)g * v.ncell;
-  double *I = (double *)a.I + (2 * tr.seg_off + (int64_t)sense * tr.nseg) * Q + q;
-  const int nseg = tr.nseg;
-  const double Iin = a.bnd[(sense ? tr.entry_minus : tr.entry_plus) * v.G + g];
-  double psi = 0.0, Bprev = 0.0;
-  double rb = 0.0, sb = 0.0;   // MOLC_BALANCE: sum of tau (d - psibar) and the magnitudes of the terms
-  for (int s = 0; s < nseg; ++s) {
-    const int64_t sgi = sense ? tr.seg_off + nseg - 1 - s : tr.seg_off + s;
-    const int cell = v.seg_cell[sgi];
-    const double len = v.seg_len[sgi], af = v.seg_afrac[sgi];
-    const double Bc = Bg[cell];
-    const double kt = kap[cell] + inv_cdt;
-    const double jump = s == 0 ? Iin - Bc : Bprev - Bc;
-    psi = s == 0 ? jump : psi + jump;
-    if constexpr (BAL) sb += fabs(jump);
-    if (v.facc) {   // Eq. (16): omega w times the intensity at the segment's upwind face
-      const int2 fc = v.seg_face[sgi];
-      double *fa = v.facc + (int64_t)(sense ? fc.y : fc.x) * kOutputs * v.G + g;
-      const double wi = pd.w * tr.width * (psi + Bc);
-      atomicAdd(fa + 0 * v.G, wi);
-      atomicAdd(fa + 1 * v.G, wi * Ox);
-      atomicAdd(fa + 2 * v.G, wi * Oy);
-      atomicAdd(fa + 3 * v.G, wi * Ox * Ox);
-      atomicAdd(fa + 4 * v.G, wi * Ox * Oy);
-      atomicAdd(fa + 5 * v.G, wi * Oy * Oy);
-    }
-    const double d = (I[(int64_t)s * Q] + (Bref[cell] - Bc)) * (inv_cdt / kt);
-    const double tau = kt * len * pd.inv_sinz;
-    const double one_m_e = -expm1(-tau);
-    const double ex = exp(-tau);
-    const double E1 = one_m_e / tau;
-    const double pin = psi;
-    const double x = pin - d;
-    const double pb = fma(x, E1, d);
-    // thin: psi_in - (psi_in - d)(1 - e^-tau), the change to the accuracy of expm1; thick: d + (psi_in - d) e^-tau,
-    // the transmitted part to the accuracy of exp
-    psi = tau < 0.5 ? fma(-x, one_m_e, pin) : fma(x, ex, d);
-    I[(int64_t)s * Q] = pb;
-    if constexpr (BAL) {
-      rb += tau * (d - pb);
-      sb += fabs(Bc + pin) + fabs(Bc + psi) + fabs(pin) + fabs(psi) + tau * (fabs(Bc + d) + fabs(Bc + pb));
-    }
-    const double wv = pd.w * af * pb;
-    double *acc = a.acc + (int64_t)cell * kOutputs * v.G + g;
-    atomicAdd(acc + 0 * v.G, wv);
-    atomicAdd(acc + 1 * v.G, wv * Ox);
-    atomicAdd(acc + 2 * v.G, wv * Oy);
-    atomicAdd(acc + 3 * v.G, wv * Ox * Ox);
-    atomicAdd(acc + 4 * v.G, wv * Ox * Oy);
-    atomicAdd(acc + 5 * v.G, wv * Oy * Oy);
-    Bprev = Bc;
-  }
-  if (BAL && nseg > 0) {
-    const double Iout = psi + Bprev;
-    ray_balance_max(v.balance, Iin - Iout + rb, sb, 1.0);
-  }
+  prep_tiles(b.v, b.a, b.L, m.y, m.z, 1 << 30, m.w != 0);
 }
 
 // ---------------------------------------------------------------------------------------------------------
@@ -466,10 +342,6 @@ __device__ __forceinline__ int2 ld_record(const int2 *p) {
 // copies visible to the other lanes and ordering the reads of a slot before its refill), and the new deviations
 // go back through the slot: each thread writes its own, the warp stores the slot's chunk in 16-byte pieces.  A thread whose track has ended leaves its part of the slot as it was copied,
 // so the padding it stores back is unchanged.
-// What an FP32 sweep adds to the segment update: nothing, the face reductions of Eq. 16 (MOLC_FACES), or the
-// per-ray balance check (MOLC_BALANCE).
-enum SweepExtra { kSweepPlain = 0, kSweepFaces = 1, kSweepBalance = 2 };
-
 // Shared memory of one FP32 sweep block: D staged steps of its 128 threads' deviations, cell-table entries and
 // B_ref differences.
 template <int NP, int D>
@@ -743,17 +615,6 @@ constexpr int kGatherBatch = kGatherPad;
 // a cell crossed by many characteristics of one pair (fine ray spacing) keeps the FP32 error of a few terms.
 constexpr int kPairRun = 8;
 
-// Eddington factors of one (cell, group) from the moments just assembled (Eq. 7 with the cell averages of
-// Eq. 15): f = N / (c E), 0 where E = 0.  The same operations as closure_cells, so molc_sweep_closure and
-// molc_sweep + molc_closure give the same bits.
-__device__ __forceinline__ void eddington_factors(const SweepArgs &a, int64_t idx, double E, double nxx, double nxy,
-                                                  double nyy) {
-  const double inv = E > 0 ? 1.0 / (a.c * E) : 0.0;
-  a.fxx[idx] = nxx * inv;
-  a.fxy[idx] = nxy * inv;
-  a.fyy[idx] = nyy * inv;
-}
-
 // Assembly of one (cell, group) from its six deviation sums D (state units; is = 1/scale):
 //   E = (B geo0 + D0 is)/c, F = D_F is, N_ab = B geo_ab + D_ab is, and B_ref := B.
 __device__ __forceinline__ void assemble_cell(const PlanView &v, const SweepArgs &a, int cell, int g,
@@ -936,40 +797,6 @@ __global__ void __launch_bounds__(128, NP <= 3 ? 7 : NP == 4 ? 8 : 5)
   const int4 m = map[blockIdx.x];
   const BatchInst &b = inst[m.x];
   moments_fp32_body<NP>(b.v, b.a, b.L, m.y, (int64_t)m.z * blockDim.x);
-}
-
-// ---------------------------------------------------------------------------------------------------------
-// finalize: cell assembly.  acc holds sum_m omega_m sum_{C(i,m)} (A/V) psibar (times Omega components);
-// the B_i part uses the geometric moments geo = sum_m omega_m sum_{C(i,m)} A/V (times Omega components).
-//   E = (B geo0 + D)/c, F = acc, N_ab = B geo_ab + acc_ab.  (The B part of F is zero by symmetry.)
-// ---------------------------------------------------------------------------------------------------------
-__global__ void finalize_kernel(PlanView v, SweepArgs a, Layout L) {
-  const double inv_c = 1.0 / a.c;
-  const double is = a.scale[1];   // accumulators are in the state's scaled units (exact power of two)
-  // one thread per cell, looping over groups: the cell's accumulator block is read contiguously (through L1)
-  // and every output [g][cell] is written coalesced across threads
-  for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < v.ncell; cell += gridDim.x * blockDim.x) {
-    const double g0v = v.geo[cell], gxx = v.geo[v.ncell + cell], gxy = v.geo[2 * (int64_t)v.ncell + cell],
-                 gyy = v.geo[3 * (int64_t)v.ncell + cell];
-    for (int g = 0; g < v.G; ++g) {
-      const int64_t idx = (int64_t)g * v.ncell + cell;
-      const int g0 = g / L.gc * L.gc, gc = L.gc;   // [chunk][cell][6][gc], as the sweeps accumulate
-      const double *ac = a.acc + (int64_t)kOutputs * g0 * v.ncell + (int64_t)cell * kOutputs * gc + (g - g0);
-      const double B = a.B[idx];
-      const double E = (B * g0v + __ldg(ac + 0 * gc) * is) * inv_c;
-      const double nxx = B * gxx + __ldg(ac + 3 * gc) * is;
-      const double nxy = B * gxy + __ldg(ac + 4 * gc) * is;
-      const double nyy = B * gyy + __ldg(ac + 5 * gc) * is;
-      a.out.E[idx] = E;
-      a.out.Fx[idx] = __ldg(ac + 1 * gc) * is;
-      a.out.Fy[idx] = __ldg(ac + 2 * gc) * is;
-      a.out.Nxx[idx] = nxx;
-      a.out.Nxy[idx] = nxy;
-      a.out.Nyy[idx] = nyy;
-      a.Bref[idx] = B;   // the new deviations refer to this step's B
-      if (a.fxx) eddington_factors(a, idx, E, nxx, nxy, nyy);
-    }
-  }
 }
 
 // f = N / (c E) per group (Eq. 7 with the cell averages of Eq. 15); <f>_E = sum_g N_g / (c sum_g E_g).
@@ -1212,24 +1039,12 @@ int grid_for(int64_t n, int block) {
 
 }  // namespace
 
-cudaError_t launch_prep(const PlanView &v, molc_precision prec, const SweepArgs &a, cudaStream_t st) {
-  Layout L = layout_for(v, prec);
-  if (prec == MOLC_FP64) L.gc = L.n_chunks = 1;   // input checks only: one group per tile row, all groups
+cudaError_t launch_prep(const PlanView &v, const SweepArgs &a, cudaStream_t st) {
+  const Layout L = layout_for(v, MOLC_FP32);
   if (L.gc > 32 || L.n_chunks > 65535) return cudaErrorInvalidConfiguration;
   const int n_tiles = (v.ncell + kPrepCells - 1) / kPrepCells;
-  const dim3 grid((unsigned)std::min(n_tiles, 152 * 16), (unsigned)(prec == MOLC_FP64 ? v.G : L.n_chunks));
-  prep_kernel<<<grid, 128, 0, st>>>(v, a, L, prec == MOLC_FP32);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_sweep_fp64(const PlanView &v, const SweepArgs &a, cudaStream_t st) {
-  const int64_t threads = v.n_tracks * 2 * (int64_t)v.G * v.n_polar;
-  const int64_t blocks = (threads + 127) / 128;
-  if (blocks > 0x7fffffff) return cudaErrorInvalidConfiguration;
-  if (v.balance)
-    sweep_fp64_kernel<true><<<(unsigned)blocks, 128, 0, st>>>(v, a);
-  else
-    sweep_fp64_kernel<false><<<(unsigned)blocks, 128, 0, st>>>(v, a);
+  const dim3 grid((unsigned)std::min(n_tiles, 152 * 16), (unsigned)L.n_chunks);
+  prep_kernel<<<grid, 128, 0, st>>>(v, a, L);
   return cudaGetLastError();
 }
 
@@ -1281,12 +1096,8 @@ cudaError_t launch_sweep_fp32(const PlanView &v, const SweepArgs &a, cudaStream_
   }
 }
 
-cudaError_t launch_finalize(const PlanView &v, molc_precision prec, const SweepArgs &a, cudaStream_t st) {
-  const Layout L = layout_for(v, prec);
-  if (prec == MOLC_FP64) {
-    finalize_kernel<<<grid_for(v.ncell, 128), 128, 0, st>>>(v, a, L);
-    return cudaGetLastError();
-  }
+cudaError_t launch_moments_fp32(const PlanView &v, const SweepArgs &a, cudaStream_t st) {
+  const Layout L = layout_for(v, MOLC_FP32);
   const int64_t blocks = (v.n_munits * L.gc + 127) / 128;
   if (blocks > 0x7fffffff || L.n_chunks > 65535) return cudaErrorInvalidConfiguration;
   const dim3 grid((unsigned)blocks, (unsigned)L.n_chunks);
