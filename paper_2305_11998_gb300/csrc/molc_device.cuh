@@ -30,6 +30,39 @@ __device__ __forceinline__ double f32_to_f64_exact(float x) {
   return (__float_as_uint(x) & 0x7f800000u) ? f32_to_f64(x) : (double)x;
 }
 
+// Exponent k of a power of two x = 2^k (a normal double).
+__device__ __forceinline__ int exponent_of(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) - 1023; }
+
+// x 2^k in FP64; by two products, as the factor itself may lie outside the normal range.  Out of line, so that the
+// integer forms below, which call it for the few values they do not take, do not execute its FP64 operations for all.
+static __device__ __noinline__ double scale_pow2_fp64(double x, int k) {
+  const double h = __hiloint2double((1023 + (k >> 1)) << 20, 0), r = __hiloint2double((1023 + k - (k >> 1)) << 20, 0);
+  return x * h * r;
+}
+
+// x 2^k as a double: integer operations where x is a normal float and the result a normal double, or x is zero.
+__device__ __forceinline__ double scaled_to_double(float x, int k) {
+  const unsigned u = __float_as_uint(x);
+  const int e = (int)((u >> 23) & 0xff), ed = e - 127 + 1023 + k;
+  if (e == 0 || e == 0xff || (unsigned)(ed - 1) >= 2046u) {
+    if ((u << 1) == 0) return __hiloint2double((int)u, 0);
+    return scale_pow2_fp64((double)x, k);
+  }
+  return __hiloint2double((int)((u & 0x80000000u) | ((unsigned)ed << 20) | ((u & 0x7fffffu) >> 3)), (int)(u << 29));
+}
+
+// x 2^k rounded to the nearest float (ties to even): integer operations where x and the float are normal, or x is zero.
+__device__ __forceinline__ float scaled_to_float(double x, int k) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ff), ef = e - 1023 + k + 127;
+  if (e == 0 || e == 0x7ff || (unsigned)(ef - 1) >= 253u) {
+    if (((hi << 1) | lo) == 0) return __uint_as_float(hi);
+    return (float)scale_pow2_fp64(x, k);
+  }
+  const unsigned f = ((hi & 0xfffffu) << 3) | (lo >> 29), rest = lo << 3;   // 23 bits, and what is cut
+  return __uint_as_float((hi & 0x80000000u) | (((unsigned)ef << 23) + f + (rest > 0x80000000u - (f & 1))));
+}
+
 // What an FP32 sweep adds to the segment update: nothing, the face reductions of Eq. 16 (MOLC_FACES), or the
 // per-ray balance check (MOLC_BALANCE).
 enum SweepExtra { kSweepPlain = 0, kSweepFaces = 1, kSweepBalance = 2 };

@@ -866,41 +866,96 @@ __global__ void closure_kernel(PlanView v, molc_moments m, double c, double *fxx
 }
 
 
-// Canonical segment averages <-> deviation state: one thread per row (track, sense, step) of the layout,
-// looping over polar cosines and the selected groups.  Ibar = B_ref(cell) + delta.
-template <class T>
-__global__ void intensity_copy_kernel(PlanView v, Layout L, T *I, const double *Bref, const double *scale,
-                                      int g_begin, int g_count, double *canon, int to_canon, int bundle) {
-  const int NP = v.n_polar;
-  const double sc = scale[0], is = scale[1];
-  for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < L.rows;
-       row += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t t = find_track(v.tracks, v.n_tracks, row);
-    const TrackDev tr = v.tracks[t];
-    const int64_t local = row - 2 * tr.seg_off;
-    const int sense = local >= tr.nseg;
-    const int s = (int)(local - (int64_t)sense * tr.nseg);
-    const int cell = v.seg_cell[sense ? tr.seg_off + tr.nseg - 1 - s : tr.seg_off + s];
-    for (int p = 0; p < NP; ++p) {
-      const PolarDev pd = v.polar[tr.pair * NP + p];
-      const int dir = sense ? pd.dir_minus : pd.dir_plus;
-      const int64_t cs = v.dir_seg_off[dir] + (sense ? tr.canon_minus : tr.canon_plus) + s;
-      for (int g = g_begin; g < g_begin + g_count; ++g) {
-        const int ch = g / L.gc, gl = g - ch * L.gc, gcount = min(L.gc, v.G - ch * L.gc);
-        T *el = bundle ? I + bundle_index(v.boff,
-                                          (int64_t)ch * 2 * v.n_tracks * L.gc +
-                                              (int64_t)tr.pos[sense] * gcount + gl,
-                                          s, NP) + p
-                       : I + L.rows * (int64_t)NP * (ch * L.gc) + row * (int64_t)(gcount * NP) + gl * NP + p;
-        const double br = Bref[(int64_t)g * v.ncell + cell];
-        double *cv = canon + cs * g_count + (g - g_begin);
-        if (to_canon)
-          *cv = br + (double)*el * is;
-        else
-          *el = (T)((*cv - br) * sc);
-      }
+// Canonical segment averages <-> deviation state, Ibar = B_ref(cell) + delta: one block per (track, sense).  The
+// canonical rows of one (track, sense, polar cosine) are contiguous, [step][selected group], so consecutive threads
+// take consecutive (step, group) pairs and, for each, the NP adjacent deviations of the state (a block reads runs of
+// groups x NP values and writes NP contiguous streams).  One thread per state row, looping over polar cosines and
+// groups, had every lane on rows of its own: 64^2 x 17 groups, 4 x 32 directions, h/4 (4.6e7 values, 0.55 GB)
+// 565 us either way; so it is 135 us out and 159 us in.  That is bound by the FP64 pipe (one addition a value, busy
+// 71 and 60 %; the power-of-two scalings and the conversions are integer operations), with DRAM at 3.5 TB/s next.
+// One thread's elements of a walk, (step, group) by (step, group): f(step, group).
+template <class F>
+__device__ __forceinline__ void for_walk(int nseg, int g_count, F f) {
+  int s = (int)threadIdx.x / g_count, gi = (int)threadIdx.x - s * g_count;
+  const int ds = (int)blockDim.x / g_count, dg = (int)blockDim.x - ds * g_count;
+  for (; s < nseg; s += ds) {
+    f(s, gi);
+    gi += dg;
+    if (gi >= g_count) {
+      gi -= g_count;
+      ++s;
     }
   }
+}
+
+template <int NP, bool TO_CANON>
+__global__ void __launch_bounds__(128) intensity_copy_fp32_kernel(PlanView v, Layout L, float *I, const double *Bref,
+                                                                  const double *scale, int g_begin, int g_count,
+                                                                  double *canon) {
+  // 1/scale and scale are powers of two
+  const double sc = scale[0], is = scale[1];
+  const int k_out = exponent_of(is), k_in = exponent_of(sc);
+  const TrackDev tr = v.tracks[blockIdx.x >> 1];
+  const int sense = blockIdx.x & 1;
+  const int pos = sense ? tr.pos[1] : tr.pos[0];
+  const int64_t cs = sense ? tr.canon_minus : tr.canon_plus;
+  double *cv[NP];
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    const PolarDev &pd = v.polar[tr.pair * NP + p];
+    cv[p] = canon + (v.dir_seg_off[sense ? pd.dir_minus : pd.dir_plus] + cs) * g_count;
+  }
+  const int *cells = v.seg_cell + (sense ? tr.seg_off + tr.nseg - 1 : tr.seg_off);
+  auto element = [&](int s, int gi, bool fast) {
+    const int g = g_begin + gi, ch = g / L.gc, gl = g - ch * L.gc, gcount = min(L.gc, v.G - ch * L.gc);
+    float *el = I + bundle_index(v.boff, (int64_t)ch * 2 * v.n_tracks * L.gc + (int64_t)pos * gcount + gl, s, NP);
+    const double br = Bref[(int64_t)g * v.ncell + cells[sense ? -s : s]];
+    const int64_t o = (int64_t)s * g_count + gi;
+    float x[NP];
+    if constexpr (TO_CANON) {
+      load_dev_cg<NP>(el, x);
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        __stcs(cv[p] + o, br + (fast ? scaled_to_double(x[p], k_out) : (double)x[p] * is));
+      }
+    } else {
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const double y = __ldcs(cv[p] + o) - br;
+        x[p] = fast ? scaled_to_float(y, k_in) : (float)(y * sc);
+      }
+#pragma unroll
+      for (int p = 0; p < NP; ++p) el[p] = x[p];
+    }
+  };
+  if (abs(k_out) < 1023 && abs(k_in) < 1023)
+    for_walk(tr.nseg, g_count, [&](int s, int gi) { element(s, gi, true); });
+  else   // a scale outside the normal range
+    for_walk(tr.nseg, g_count, [&](int s, int gi) { element(s, gi, false); });
+}
+
+// The FP64 state: rows (track, sense, step) of [G][NP].
+template <bool TO_CANON>
+__global__ void __launch_bounds__(128) intensity_copy_fp64_kernel(PlanView v, double *I, const double *Bref, int g_begin,
+                                                                  int g_count, double *canon) {
+  const int NP = v.n_polar;
+  const TrackDev tr = v.tracks[blockIdx.x >> 1];
+  const int sense = blockIdx.x & 1;
+  const int64_t cs = sense ? tr.canon_minus : tr.canon_plus;
+  const int *cells = v.seg_cell + (sense ? tr.seg_off + tr.nseg - 1 : tr.seg_off);
+  for_walk(tr.nseg, g_count, [&](int s, int gi) {
+    const int g = g_begin + gi;
+    double *el = I + ((2 * tr.seg_off + (int64_t)sense * tr.nseg + s) * v.G + g) * NP;
+    const double br = Bref[(int64_t)g * v.ncell + cells[sense ? -s : s]];
+    for (int p = 0; p < NP; ++p) {
+      const PolarDev &pd = v.polar[tr.pair * NP + p];
+      double *cv = canon + (v.dir_seg_off[sense ? pd.dir_minus : pd.dir_plus] + cs + s) * g_count + gi;
+      if constexpr (TO_CANON)
+        __stcs(cv, br + el[p]);
+      else
+        el[p] = __ldcs(cv) - br;
+    }
+  });
 }
 
 // max over finite non-negative B of the IEEE bits (ordered like the values for x >= 0)
@@ -1261,12 +1316,34 @@ cudaError_t launch_intensity_copy(const PlanView &v, molc_precision prec, void *
                                   const double *scale, int g_begin, int g_count, double *canon, bool to_canon,
                                   cudaStream_t st) {
   const Layout L = layout_for(v, prec);
-  if (prec == MOLC_FP64)
-    intensity_copy_kernel<double><<<grid_for(L.rows, 128), 128, 0, st>>>(v, L, (double *)I, Bref, scale, g_begin,
-                                                                         g_count, canon, to_canon, 0);
-  else
-    intensity_copy_kernel<float><<<grid_for(L.rows, 128), 128, 0, st>>>(v, L, (float *)I, Bref, scale, g_begin,
-                                                                       g_count, canon, to_canon, 1);
+  if (v.n_tracks > 0x3fffffff) return cudaErrorInvalidConfiguration;
+  const unsigned blocks = (unsigned)(2 * v.n_tracks);
+  if (prec == MOLC_FP64) {
+    if (to_canon)
+      intensity_copy_fp64_kernel<true><<<blocks, 128, 0, st>>>(v, (double *)I, Bref, g_begin, g_count, canon);
+    else
+      intensity_copy_fp64_kernel<false><<<blocks, 128, 0, st>>>(v, (double *)I, Bref, g_begin, g_count, canon);
+    return cudaGetLastError();
+  }
+  switch (v.n_polar) {
+#define MOLC_COPY(NP)                                                                                                  \
+  case NP:                                                                                                             \
+    if (to_canon)                                                                                                      \
+      intensity_copy_fp32_kernel<NP, true><<<blocks, 128, 0, st>>>(v, L, (float *)I, Bref, scale, g_begin, g_count, canon); \
+    else                                                                                                               \
+      intensity_copy_fp32_kernel<NP, false><<<blocks, 128, 0, st>>>(v, L, (float *)I, Bref, scale, g_begin, g_count, canon); \
+    break;
+    MOLC_COPY(1)
+    MOLC_COPY(2)
+    MOLC_COPY(3)
+    MOLC_COPY(4)
+    MOLC_COPY(5)
+    MOLC_COPY(6)
+    MOLC_COPY(7)
+    MOLC_COPY(8)
+#undef MOLC_COPY
+    default: return cudaErrorInvalidValue;
+  }
   return cudaGetLastError();
 }
 
