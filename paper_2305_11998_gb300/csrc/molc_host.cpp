@@ -105,12 +105,15 @@ struct molc_plan {
   Cell64 *d_cell64 = nullptr;
   int2 *d_items32 = nullptr;
   int64_t n_items32 = 0;
-  int64_t *d_cell_off = nullptr;
-  int4 *d_gent = nullptr;
+  int64_t *d_unit_off = nullptr;
+  GatherRun *d_gent = nullptr;
+  float *d_fold = nullptr;
   int64_t *d_boff = nullptr;
   int2 *d_seg_face = nullptr;
   unsigned long long *d_balance = nullptr;   // MOLC_BALANCE: largest per-ray relative residual (double bits)
   int2 *d_munit = nullptr;
+  int batch_munit[2] = {1, 1};   // FP32 moments in a batch: units of a block (as PlanView::munit_block), its shared memory
+  size_t batch_msmem = 0;
   int4 *d_mmulti = nullptr;
   double *d_mscratch = nullptr;
   double *d_facc = nullptr;
@@ -364,7 +367,7 @@ void free_device(molc_plan *p) {
   free_events(p);
   void *ptrs[] = {p->d_tracks, p->d_seg32, p->d_seg_cell, p->d_seg_len, p->d_seg_afrac, p->d_pairs, p->d_polar,
                   p->d_geo, p->d_dir_seg_off, p->d_status, p->d_cdat, p->d_cdB, p->d_acc, p->d_items32,
-                  p->d_cell_off, p->d_gent, p->d_boff, p->d_block_order, p->d_seg_face, p->d_facc,
+                  p->d_unit_off, p->d_gent, p->d_fold, p->d_boff, p->d_block_order, p->d_seg_face, p->d_facc,
                   p->d_munit, p->d_mmulti, p->d_mscratch, p->d_balance, p->d_polar_fix, p->d_cell64, p->d_track_order};
   for (void *q : ptrs)
     if (q) cudaFree(q);
@@ -704,6 +707,18 @@ std::string device_signature(int dev) {
   char buf[320];
   std::snprintf(buf, sizeof buf, "%s, %d SMs, sm_%d%d", pr.name, pr.multiProcessorCount, pr.major, pr.minor);
   return buf;
+}
+
+// Units a block of the moment gather takes in a chunk of gcount groups (no more than leave `blocks` blocks), and its
+// shared memory.
+int moment_units(const std::vector<int64_t> &unit_off, int gcount, int64_t blocks, size_t &smem) {
+  const int64_t n = (int64_t)unit_off.size() - 1;
+  for (int units = (int)std::max<int64_t>(1, std::min<int64_t>(kMomentBlock / gcount, n / blocks));; --units) {
+    int64_t most = 0;
+    for (int64_t u = 0; u < n; u += units) most = std::max(most, unit_off[std::min(n, u + units)] - unit_off[u]);
+    smem = moment_smem(most, gcount);
+    if (units == 1 || smem <= kMomentSmem) return units;
+  }
 }
 
 }  // namespace
@@ -1154,77 +1169,113 @@ molc_status molc_create(const molc_grid *grid, const molc_quadrature *quad, cons
   p->bundle_slots = boff[n_blocks32];
   p->n_blocks32 = n_blocks32;
 
-  // ---- FP32 cell moments are gathered per cell from the swept state: for every cell, one entry per (track,
-  // sense) segment crossing it, {item position of the (track, sense), step along that sense, A/V (f32 bits),
-  // 2 pair + sense}; the + sense reaches the track's j-th segment at step j, the - sense at step nseg - 1 - j.
-  // Entries of a cell are in track order (so grouped by azimuth pair), and the gathered sums deterministic.
+  // ---- FP32 cell moments are gathered per cell from the swept state: for every cell, the item position and step
+  // of both senses of each track segment crossing it; the + sense reaches the track's j-th segment at step j, the
+  // - sense at step nseg - 1 - j.  The segments of a cell are in track order (so grouped by azimuth pair), and the
+  // gathered sums deterministic.
   if (2 * S > (int64_t)0x7fffffff) {
     delete p;
     return fail(MOLC_ERR_INVALID_ARG, "create: too many segments for the FP32 state rows");
   }
-  // Each cell's list is padded to a multiple of kGatherPad entries with zero-area copies of its last entry.
   if ((size_t)p->n_pairs * (3 * p->n_polar + 2) * sizeof(float) > kMaxGatherSmem) {
     delete p;
     return fail(MOLC_ERR_INVALID_ARG, "create: too many azimuth pairs for the FP32 moment kernel");
   }
-  std::vector<int64_t> cell_off(nch32 ? (size_t)ncell + 1 : 0, 0);
-  std::vector<int4> gent;
+  // A unit of the gather is a cell, or a part of kPartSegments segments of a cell that more segments cross (fine ray
+  // spacing); the parts of such a cell are added in order by a second kernel (deterministic).  A unit's segments are
+  // cut into runs of up to kRunSegments of one pair.
+  std::vector<int64_t> unit_off(nch32 ? 1 : 0, 0);
+  std::vector<GatherRun> gent;
+  std::vector<int2> munit;
+  std::vector<int4> mmulti;
+  int64_t n_munits = 0;
   if (nch32) {
-    std::vector<int64_t> cnt(ncell, 0);
-    for (int64_t q = 0; q < S; ++q) cnt[p->seg_cell[q]] += 2;
-    for (int i = 0; i < ncell; ++i) cell_off[i + 1] = cell_off[i] + (cnt[i] + kGatherPad - 1) / kGatherPad * kGatherPad;
-    gent.assign((size_t)cell_off[ncell], make_int4(0, 0, 0, 0));
-    std::vector<int64_t> pos(cell_off.begin(), cell_off.end() - 1);
-    // in parallel over ranges of cells: every range scans all tracks in order and writes its own cells' entries,
-    // so each list is in track order as from one serial scan
-    const int64_t n_ranges = std::min<int64_t>(ncell, 4 * (int64_t)std::max(1u, std::thread::hardware_concurrency()));
-    parallel_for(n_ranges, [&](int64_t r) {
-      const int c_lo = (int)(ncell * r / n_ranges), c_hi = (int)(ncell * (r + 1) / n_ranges);
-      for (int64_t k = 0; k < T; ++k) {
-        const TrackDev &t = td[k];
-        for (int j = 0; j < t.nseg; ++j) {
-          const int64_t q = t.seg_off + j;
-          const int c = p->seg_cell[q];
-          if (c < c_lo || c >= c_hi) continue;
-          const float af = (float)p->seg_afrac[q];
-          int afb;
-          std::memcpy(&afb, &af, 4);
-          gent[pos[c]++] = make_int4(t.pos[0], j, afb, 2 * t.pair);
-          gent[pos[c]++] = make_int4(t.pos[1], t.nseg - 1 - j, afb, 2 * t.pair + 1);
-        }
+    struct Filling {   // a cell's list while the tracks are scanned: its segments and runs, its last run
+      int segs = 0, pair = -1, in_run = 0;
+      int64_t runs = 0;
+      // whether the next segment, of pair `pr`, begins a run (and a unit)
+      bool next(int pr) {
+        const bool fresh = segs % kPartSegments == 0 || pr != pair || in_run == kRunSegments;
+        in_run = fresh ? 1 : in_run + 1;
+        pair = pr;
+        ++segs;
+        runs += fresh;
+        return fresh;
       }
-      for (int i = c_lo; i < c_hi; ++i)
-        for (int64_t e = pos[i]; e < cell_off[i + 1]; ++e) {
-          gent[e] = gent[pos[i] - 1];
-          gent[e].z = 0;   // zero area
+    };
+    std::vector<Filling> fill(ncell);
+    // in parallel over ranges of cells: every range scans all tracks in order and takes its own cells' segments, so
+    // each list is in track order as from one serial scan
+    const int64_t n_ranges =
+        big ? std::min<int64_t>(ncell, (int64_t)std::max(1u, std::thread::hardware_concurrency())) : 1;
+    auto for_segments = [&](auto take) {   // take(cell, track, segment of the track)
+      parallel_for(n_ranges, [&](int64_t r) {
+        const int c_lo = (int)(ncell * r / n_ranges), c_hi = (int)(ncell * (r + 1) / n_ranges);
+        for (int64_t k = 0; k < T; ++k) {
+          const TrackDev &t = td[k];
+          const int *cells = &p->seg_cell[t.seg_off];
+          for (int j = 0; j < t.nseg; ++j)
+            if (cells[j] >= c_lo && cells[j] < c_hi) take(cells[j], t, j);
         }
-    }, big);
-    // Per chunk, the (item position, step) of each entry becomes the state slot of the chunk's group 0 plus the
-    // bundle length and lane (gather_slot); chunks 1.. are written from the chunk-0 list first, chunk 0 last,
-    // in place.
-    const int64_t n_ent = cell_off[ncell];
-    gent.resize((size_t)(n_ent * nch32));
+      }, big);
+    };
+    for_segments([&](int c, const TrackDev &t, int) { fill[c].next(t.pair); });
+    std::vector<int64_t> pos(ncell), first_unit(ncell);   // next run of a cell, its first unit
+    int64_t n_run = 0;
+    bool split = false;
+    for (int i = 0; i < ncell; ++i) {
+      const int parts = std::max(1, (fill[i].segs + kPartSegments - 1) / kPartSegments);
+      pos[i] = n_run;
+      first_unit[i] = (int64_t)munit.size();
+      if (parts > 1) mmulti.push_back(make_int4(i, (int)munit.size(), parts, 0));
+      split |= parts > 1;
+      for (int k = 0; k < parts; ++k) munit.push_back(make_int2(i, parts));
+      n_run += fill[i].runs;
+      unit_off.resize(munit.size() + 1, n_run);   // but for the units of a split cell: below
+      fill[i] = Filling();
+    }
+    n_munits = (int64_t)munit.size();
+    if (!split) munit.clear();
+    gent.resize((size_t)(n_run * nch32));
+    for_segments([&](int c, const TrackDev &t, int j) {
+      if (fill[c].segs % kPartSegments == 0) unit_off[first_unit[c] + fill[c].segs / kPartSegments] = pos[c];
+      if (fill[c].next(t.pair)) gent[pos[c]++] = GatherRun{};
+      GatherRun &run = gent[pos[c] - 1];
+      run.seg[run.count] = make_int4(t.pos[0], t.pos[1], j, t.nseg - 1 - j);   // item positions and steps for now
+      run.area[run.count] = (float)p->seg_afrac[t.seg_off + j];
+      run.pair = t.pair;
+      run.cf = p->pairs[t.pair].cf;
+      run.sf = p->pairs[t.pair].sf;
+      ++run.count;
+    });
+    // Per chunk, the (item position, step) of each segment and sense becomes the state slot of the chunk's group 0
+    // plus the bundle length and lane (gather_slot); chunks 1.. are written from the chunk-0 list first, chunk 0
+    // last, in place.
     std::atomic<bool> too_large(false);
     for (int ch = nch32 - 1; ch >= 0; --ch) {
       const int gcount = std::min(gc32, p->G - ch * gc32);
       const int64_t item_base = (int64_t)ch * 2 * T * gc32;
-      const int64_t n_blocks = (n_ent + 65535) / 65536;   // entries in blocks of 64 Ki, in parallel
+      const int64_t n_blocks = (n_run + 16383) / 16384;   // runs in blocks of 16 Ki, in parallel
       parallel_for(n_blocks, [&](int64_t blk) {
-        const int64_t e1 = std::min(n_ent, (blk + 1) * 65536);
-        for (int64_t e = blk * 65536; e < e1; ++e) {
-          int4 r = gent[e];
-          const int64_t item = item_base + (int64_t)r.x * gcount;
+        const int64_t e1 = std::min(n_run, (blk + 1) * 16384);
+        auto place = [&](int &x, int &y) {   // item position and step -> slot words
+          const int64_t item = item_base + (int64_t)x * gcount;
           const int64_t b = item / kSweepBlock;
           const int lane = (int)(item % kSweepBlock);
-          const int64_t slot = (boff[b] + r.y) * kSweepBlock + lane;
+          const int64_t slot = (boff[b] + y) * kSweepBlock + lane;
           const int64_t blen = boff[b + 1] - boff[b];
-          if ((slot >> (32 + (32 - kGatherSlotHiShift))) != 0 || blen > (int64_t)kGatherBlenMask) {
-            too_large = true;
-            return;
-          }
-          r.x = (int)(uint32_t)(slot & 0xffffffffLL);
-          r.y = (int)(((uint32_t)(slot >> 32) << kGatherSlotHiShift) | ((uint32_t)blen << 7) | (uint32_t)lane);
-          gent[(size_t)(ch * n_ent + e)] = r;
+          x = (int)(uint32_t)(slot & 0xffffffffLL);
+          y = (int)(((uint32_t)(slot >> 32) << kGatherSlotHiShift) | ((uint32_t)blen << 7) | (uint32_t)lane);
+          return (slot >> (32 + (32 - kGatherSlotHiShift))) == 0 && blen <= (int64_t)kGatherBlenMask;
+        };
+        for (int64_t e = blk * 16384; e < e1; ++e) {
+          GatherRun r = gent[e];
+          for (int i = 0; i < r.count; ++i)
+            if (!place(r.seg[i].x, r.seg[i].z) || !place(r.seg[i].y, r.seg[i].w)) {
+              too_large = true;
+              return;
+            }
+          gent[(size_t)(ch * n_run + e)] = r;
         }
       }, big);
       if (too_large) {
@@ -1233,18 +1284,19 @@ molc_status molc_create(const molc_grid *grid, const molc_quadrature *quad, cons
       }
     }
   }
-  // Work units of the moment gather: each cell's entry list in parts of at most kPartEntries entries, so that a
-  // cell crossed by very many characteristics (fine ray spacing) is summed by several threads; the parts of a
-  // split cell are added in order by a second kernel (deterministic).
-  std::vector<int2> munit;
-  std::vector<int4> mmulti;
+  // coefficients of the gather
+  std::vector<float> fold;
   if (nch32) {
-    static_assert(kPartEntries % kGatherPad == 0, "parts must hold whole gather batches");
-    for (int i = 0; i < ncell; ++i) {
-      const int64_t n = cell_off[i + 1] - cell_off[i];
-      const int parts = (int)std::max<int64_t>(1, (n + kPartEntries - 1) / kPartEntries);
-      if (parts > 1) mmulti.push_back(make_int4(i, (int)munit.size(), parts, 0));
-      for (int k = 0; k < parts; ++k) munit.push_back(make_int2(i, k));
+    const int row = fold_row(p->n_polar), stride = fold_stride(p->n_polar);
+    fold.assign((size_t)p->n_pairs * stride, 0.f);
+    for (int j = 0; j < p->n_pairs; ++j) {
+      float *f = &fold[(size_t)j * stride];
+      for (int k = 0; k < p->n_polar; ++k) {
+        const PolarDev &pd = p->polar[(size_t)j * p->n_polar + k];
+        f[k] = pd.wf;
+        f[row + k] = pd.wf * pd.sinzf;
+        f[2 * row + k] = f[row + k] * pd.sinzf;
+      }
     }
   }
   p->n_split_cells = (int)mmulti.size();
@@ -1324,13 +1376,14 @@ molc_status molc_create(const molc_grid *grid, const molc_quadrature *quad, cons
   UP(d_geo, geo.data(), geo.size(), "geometric moments")
   UP(d_dir_seg_off, p->dir_seg_off.data(), p->dir_seg_off.size(), "direction offsets")
   UP(d_status, (const int *)nullptr, 1, "status")
-  UP(d_cell_off, cell_off.data(), cell_off.size(), "cell entry offsets")
+  UP(d_unit_off, unit_off.data(), unit_off.size(), "moment units")
   UP(d_gent, gent.data(), gent.size(), "cell entries")
+  UP(d_fold, fold.data(), fold.size(), "cell entries")
   UP(d_boff, boff.data(), boff.size(), "state bundles")
   UP(d_seg_face, seg_face.data(), seg_face.size(), "segment faces")
   UP(d_munit, munit.data(), munit.size(), "moment units")
   UP(d_mmulti, mmulti.data(), mmulti.size(), "split cells")
-  UP(d_mscratch, (const double *)nullptr, mmulti.empty() ? 0 : (size_t)nch32 * munit.size() * kOutputs * gc32,
+  UP(d_mscratch, (const double *)nullptr, mmulti.empty() ? 0 : (size_t)nch32 * n_munits * kOutputs * gc32,
      "moment partials")
   UP(d_facc, (const double *)nullptr, p->facc_elems, "face accumulators")
   UP(d_balance, (const unsigned long long *)nullptr, (flags & MOLC_BALANCE) ? 2 : 0, "balance residual")
@@ -1363,15 +1416,25 @@ molc_status molc_create(const molc_grid *grid, const molc_quadrature *quad, cons
   v.geo = p->d_geo;
   v.dir_seg_off = p->d_dir_seg_off;
   v.status = p->d_status;
-  v.cell_off = p->d_cell_off;
+  v.unit_off = p->d_unit_off;
   v.gent = p->d_gent;
-  v.gent_chunk = nch32 ? cell_off[ncell] : 0;
+  v.gent_chunk = nch32 ? unit_off.back() : 0;
+  v.fold = p->d_fold;
   v.boff = p->d_boff;
   v.block_order = p->d_block_order;
   v.seg_face = p->d_seg_face;
   v.facc = p->d_facc;
   v.munit = p->d_munit;
-  v.n_munits = (int64_t)munit.size();
+  v.n_munits = n_munits;
+  if (nch32)
+    for (int last = 0; last < 2; ++last) {
+      const int gcount = last && p->G % gc32 ? p->G % gc32 : gc32;
+      size_t smem = 0;
+      v.munit_block[last] = moment_units(unit_off, gcount, kMomentBlocks, smem);
+      v.msmem = std::max(v.msmem, smem);
+      p->batch_munit[last] = moment_units(unit_off, gcount, 1, smem);
+      p->batch_msmem = std::max(p->batch_msmem, smem);
+    }
   v.mmulti = p->d_mmulti;
   v.n_mmulti = (int)mmulti.size();
   v.mscratch = p->d_mscratch;
@@ -2014,12 +2077,14 @@ molc_status molc_batch_create(molc_plan *const *plans, int n, molc_batch **out) 
     auto &m = mo[p->n_polar];
     for (int ch = 0; ch < L.n_chunks; ++ch) {
       const int gcount = std::min(L.gc, v.G - ch * L.gc);
-      const int64_t nb = (v.n_munits * gcount + 127) / 128;
-      for (int64_t k = 0; k < nb; ++k) m.push_back(make_int4(i, ch, (int)k, 0));
+      // the launch's blocks are many together: as many units a block as it holds
+      const int units = p->batch_munit[gcount == L.gc ? 0 : 1];
+      const int64_t nb = moment_blocks(v, units);
+      for (int64_t k = 0; k < nb; ++k) m.push_back(make_int4(i, ch, (int)k, units));
       const int64_t nc = ((int64_t)v.n_mmulti * gcount + 127) / 128;
       for (int64_t k = 0; k < nc; ++k) comb.push_back(make_int4(i, ch, (int)k, 0));
     }
-    mo_smem[p->n_polar] = std::max(mo_smem[p->n_polar], (size_t)v.n_pairs * (3 * v.n_polar + 2) * sizeof(float));
+    mo_smem[p->n_polar] = std::max(mo_smem[p->n_polar], p->batch_msmem);
   }
   cudaError_t e = cudaMalloc((void **)&b->d_inst, n * sizeof(BatchInst));
   if (e == cudaSuccess) e = upload_vec(&b->d_prep, prep);

@@ -10,10 +10,18 @@ namespace molc {
 
 constexpr int kMaxPolarFP32 = 8;     // FP32 sweep: polar cosines per azimuth handled by one half-warp
 constexpr int kOutputs = 6;          // D, Fx, Fy, Nxx, Nxy, Nyy accumulators per (cell, group)
-constexpr int kGatherPad = 4;        // FP32 moments: each cell's entry list is padded to a multiple of this
-constexpr int kPartEntries = 256;    // FP32 moments: entries one thread sums (longer cell lists are split)
+constexpr int kPartSegments = 128;   // FP32 moments: segments of a cell summed as one unit (longer lists are split)
+constexpr int kMomentBlock = 128;    // FP32 moments: threads of a block
+// A block of the gather takes as many units as give its second phase, one thread per (unit, group), a thread each, but
+// leaves 24 blocks to an SM where there are so many units (64^2 x 17 groups: 157 us a step with 8, 137 with 24), and no
+// more than 22 KB of runs and sums: 7 blocks to an SM beside an L1 that still holds the coefficients and parameters
+// (512^2 x 17 groups, 4 polar cosines 3425 us a step with 28 KB, 3414 with 22, 3464 with 16; 160 x 120 x 17 groups, 3
+// polar cosines 423, 367, 371).  A single unit may take more: at most kPartSegments runs, 61 KB with 32 groups.
+constexpr int64_t kMomentBlocks = 152 * 24;
+constexpr size_t kMomentSmem = 22 * 1024;
+constexpr int kRunSegments = 4;      // FP32 moments: segments of one azimuth pair summed in FP32 (GatherRun)
 constexpr int kSweepBlock = 128;     // FP32 sweep: work items (threads) per block = width of a state bundle
-constexpr size_t kMaxGatherSmem = 200 * 1024;  // FP32 moments: per-pair coefficient table in shared memory
+constexpr size_t kMaxGatherSmem = 200 * 1024;  // FP32: the per-pair coefficients a plan may have, in bytes
 
 // Device status bits (the first one set wins in molc_device_status).
 constexpr int kStatusNonfinite = 1;
@@ -61,6 +69,20 @@ struct alignas(32) Cell64 {
   double kt, r, B, dB;
 };
 
+// FP32 moments: up to kRunSegments track segments of one azimuth pair that cross a cell, in track order.  seg: of each,
+// {state slot of group 0 of the chunk, bits 0-31, for the + sense, for the - sense, and for each {slot bits 32-36 << 27 |
+// bundle length << 7 | lane} (gather_slot)}; the areas A/V; the pair, its cos and sin, and the
+// number of segments.
+struct alignas(16) GatherRun {
+  int4 seg[kRunSegments];
+  float area[kRunSegments];
+  int pair, count;
+  float cf, sf;
+};
+// Per azimuth pair, the gather's coefficients: w, w sin and w sin^2 of its polar cosines, each row padded to vector loads.
+__host__ __device__ constexpr int fold_row(int np) { return np <= 2 ? 2 : (np + 3) / 4 * 4; }
+__host__ __device__ constexpr int fold_stride(int np) { return 3 * fold_row(np); }
+
 // Everything a kernel needs, by value.
 struct PlanView {
   int nx, ny, ncell, G, n_pairs, n_polar;
@@ -78,13 +100,14 @@ struct PlanView {
   const int64_t *dir_seg_off;   // canonical segment offset of each direction
   int *status;
   int gc32;                     // FP32 sweep: groups per chunk
-  const int64_t *cell_off;      // FP32 moments: [ncell + 1] offsets into one chunk's gent entries
-  const int4 *gent;             // FP32 moments: [chunk][entry] {state slot bits 0-31, slot bits 32-36 << 27 |
-                                //   bundle length << 7 | lane, A/V f32 bits, 2 pair + sense} (gather_slot)
-  int64_t gent_chunk;           // FP32 moments: entries per chunk (cell_off[ncell])
-  const int2 *munit;            // FP32 moments: work units {cell, part}, cell-major; part k sums the cell's entries
-                                //   [kPartEntries k, kPartEntries (k + 1))
+  const int64_t *unit_off;      // FP32 moments: [n_munits + 1] offsets of the units into one chunk's runs
+  const GatherRun *gent;        // FP32 moments: [chunk][run]
+  int64_t gent_chunk;           // FP32 moments: runs per chunk
+  const float *fold;            // FP32 moments: [pair][3][fold_row] coefficients
+  const int2 *munit;            // FP32 moments: units {cell, parts of the cell}, cell-major, or null: one unit a cell
   int64_t n_munits;
+  int munit_block[2];           // FP32 moments: units a block takes in a chunk of gc32 groups, in a smaller last one
+  size_t msmem;                 // FP32 moments: dynamic shared memory of a block
   const int4 *mmulti;           // FP32 moments: cells split in more than one part: {cell, first unit, parts, 0}
   int n_mmulti;
   double *mscratch;             // FP32 moments: [chunk][unit][6][gc] partial sums of split cells (or null)
@@ -111,18 +134,24 @@ __host__ __device__ inline int64_t bundle_index(const int64_t *boff, int64_t ite
   return ((boff[item / kSweepBlock] + s) * kSweepBlock + item % kSweepBlock) * NP;
 }
 
-// A moment-gather entry addresses the state slot of group 0 of its chunk directly: slot = (boff[b] + step) 128
+// A moment-gather run addresses the state slot of group 0 of its chunk directly: slot = (boff[b] + step) 128
 // + lane for the item of group 0 at lane `lane` of bundle b.  Group gi of the same (track, sense) is item + gi:
 // the same bundle while lane + gi < 128, else lane + gi - 128 of bundle b + 1, which starts blen(b) slots of
 // 128 later.  Packing limits (checked by the planner): slot < 2^37, bundle length < 2^20.
 constexpr int kGatherSlotHiShift = 27;
 constexpr unsigned kGatherBlenMask = 0xFFFFFu;
 __host__ __device__ inline int64_t gather_slot(int ex, int ey, int gi) {
+  static_assert(kSweepBlock == 128, "bundle length << 7 is the length in slots");
   const unsigned y = (unsigned)ey;
-  int64_t slot = (int64_t)(((uint64_t)(y >> kGatherSlotHiShift) << 32) | (unsigned)ex) + gi;
-  if ((int)(y & (kSweepBlock - 1)) + gi >= kSweepBlock)
-    slot += ((int64_t)((y >> 7) & kGatherBlenMask) - 1) * kSweepBlock;
-  return slot;
+  const unsigned ahead =
+      (unsigned)gi + ((int)(y & (kSweepBlock - 1)) + gi >= kSweepBlock ? (y & (kGatherBlenMask << 7)) - kSweepBlock : 0u);
+  return (int64_t)((((uint64_t)(y >> kGatherSlotHiShift) << 32) | (unsigned)ex) + ahead);
+}
+
+// Blocks of the moment gather over one chunk, and the shared memory of one: the runs and three sums a run and group.
+inline int64_t moment_blocks(const PlanView &v, int units) { return (v.n_munits + units - 1) / units; }
+inline size_t moment_smem(int64_t runs, int gcount) {
+  return (size_t)runs * (sizeof(GatherRun) + 3 * sizeof(float) * gcount);
 }
 
 // Group tiling of the opaque intensity state: groups are tiled in chunks of `gc` groups.  FP64 state: within a

@@ -592,14 +592,24 @@ __global__ void __launch_bounds__(kSweepBlock) sweep_fp32_batch_kernel(const Bat
   sweep_fp32_body<NP, D>(b.v, b.a, b.L, m.y, sm);
 }
 
-// FP32 path, cell moments: one thread per (chunk, cell, group), consecutive groups of a cell in consecutive
-// lanes.  The thread sums, over the (track, sense) segments crossing its cell, the swept deviations of its group
-// (NP contiguous values per segment; the lanes of a cell read one contiguous block) weighted by
-// omega (A/V) (1, Omega, Omega Omega).  A cell's entries come grouped by azimuth pair: within a pair the
-// polar folds S0 = sum_p w_p dev_p, S1 = sum_p w_p sin(zeta_p) dev_p (signed by the sense),
-// S2 = sum_p w_p sin^2(zeta_p) dev_p are summed in FP32 (runs of at most kPairRun segments); across runs the six sums
-// are carried as unevaluated pairs of FP32 words (hi + lo, TwoSum: a 48-bit significand), then assembled in FP64:
+// FP32 path, cell moments, in two phases.  A cell's (track, sense) segments come as runs of up to kRunSegments track
+// segments of one azimuth pair.  First each (run, group) is summed by a thread, in FP32: over the run's segments and
+// their two senses, the polar folds S0 = sum_p w_p dev_p, S1 = sum_p w_p sin(zeta_p) dev_p, S2 = sum_p w_p
+// sin^2(zeta_p) dev_p of the swept deviations times A/V (S1 signed by the sense).  Then each (cell, group) adds its
+// runs' three sums, times (1, Omega, Omega Omega), as unevaluated pairs of FP32 words (hi + lo, TwoSum: a 48-bit
+// significand), assembled in FP64:
 //   E = (B geo0 + D)/c, F = D_F, N_ab = B geo_ab + D_ab, and B_ref := B.
+// Memory latency bounds it: the pieces of a cell (the groups of one segment and sense, contiguous in the state) lie all
+// over the state.  With one thread walking a (cell, group)'s list, four pieces at a time, a step's loads waited for that
+// step's list words; the lanes of a warp, 2-3 cells, added their pairs' sums at different steps, so that a warp issued
+// 146 instructions per segment; and 64^2 cells x 17 groups left half the SMs' slots empty.  So a run's loads, up to eight
+// a thread, depend on nothing but words already in shared memory, the runs of a cell are spread over the block, and the
+// second phase adds in step.  The FP32 sums run over the same terms in the same order as one thread's walk (run by run,
+// segment by segment, + sense before - sense), so the moments do not depend on how cells and runs are shared out.
+// A step, before and after (the gather alone is what changed): 512^2 x 17 groups, 4 polar cosines, h/2 3523 -> 3414 us;
+// 128^2 x 17, 8 polar cosines x 64, h/8 3035 -> 2818; 64^2 x 17, 4, h/4 154 -> 137; 160 x 120 x 17, 3, h/3 391 -> 367,
+// 1 polar cosine 128^2 x 17, h/2 186 -> 172; 6 polar cosines 427 -> 428; 40^2 paper layout at 1e-3 cm 2191 -> 2091;
+// 16^2 x 4 groups 34.5 -> 28; a batch of 16 problems of 32^2 to 256^2 3709 -> 3593.
 __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float x) {
   const float s = __fadd_rn(hi, x);
   const float bp = __fsub_rn(s, hi);
@@ -608,10 +618,7 @@ __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float x) {
   lo = __fadd_rn(lo, e);
 }
 
-// Entries are taken kGatherBatch at a time so that their state loads are in flight together (each cell's entry
-// list is padded to a multiple of kGatherPad with zero-area entries of its last pair, so the batch must equal it).
-constexpr int kGatherBatch = kGatherPad;
-// An FP32 partial sum takes at most kPairRun entries (one azimuth pair) before it is added to the two-word sums:
+// Tiled sweep: an FP32 partial sum takes at most kPairRun entries (one azimuth pair) before it is added to the two-word sums:
 // a cell crossed by many characteristics of one pair (fine ray spacing) keeps the FP32 error of a few terms.
 constexpr int kPairRun = 8;
 
@@ -636,120 +643,197 @@ __device__ __forceinline__ void assemble_cell(const PlanView &v, const SweepArgs
   if (a.fxx) eddington_factors(a, idx, E, nxx, nxy, nyy);
 }
 
-// One block: threads t0 .. t0+127 of chunk ch ((unit, group) pairs, groups fastest; a unit is one part of a
-// cell's entry list).  A cell in one part is assembled here; the parts of a split cell go to the scratch
-// partials, summed in order by moments_combine.
+// Two FP32 values side by side: one instruction rounds both (sm_100+).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 x) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(x));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {   // a - b, rounded once
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(pack2(-1.f, -1.f)), "l"(a));
+  return r;
+}
+__device__ __forceinline__ void two_sum_add2(f32x2 &hi, f32x2 &lo, f32x2 x) {   // two_sum_add on each half
+  const f32x2 s = add2(hi, x);
+  const f32x2 bp = sub2(s, hi);
+  const f32x2 e = add2(sub2(hi, sub2(s, bp)), sub2(x, bp));
+  hi = s;
+  lo = add2(lo, e);
+}
+
+// load_dev_cg where `on`, else zeros.
+template <int NP>
+__device__ __forceinline__ void load_dev_if(bool on, const float *p, float (&v)[NP]) {
+#pragma unroll
+  for (int i = 0; i < NP; ++i) v[i] = 0.f;
+  if constexpr (NP % 4 == 0) {
+#pragma unroll
+    for (int i = 0; i < NP; i += 4)
+      asm("{.reg .pred q;\n setp.ne.s32 q, %5, 0;\n @q ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];}"
+          : "+f"(v[i]), "+f"(v[i + 1]), "+f"(v[i + 2]), "+f"(v[i + 3])
+          : "l"(p + i), "r"((int)on) : "memory");
+  } else if constexpr (NP % 2 == 0) {
+#pragma unroll
+    for (int i = 0; i < NP; i += 2)
+      asm("{.reg .pred q;\n setp.ne.s32 q, %3, 0;\n @q ld.global.cg.v2.f32 {%0, %1}, [%2];}"
+          : "+f"(v[i]), "+f"(v[i + 1])
+          : "l"(p + i), "r"((int)on) : "memory");
+  } else {
+#pragma unroll
+    for (int i = 0; i < NP; ++i)
+      asm("{.reg .pred q;\n setp.ne.s32 q, %2, 0;\n @q ld.global.cg.f32 %0, [%1];}"
+          : "+f"(v[i])
+          : "l"(p + i), "r"((int)on) : "memory");
+  }
+}
+
+// N consecutive coefficients, vector loads where a row is padded for them.
+template <int NP>
+__device__ __forceinline__ void load_fold(const float *p, float (&c)[NP]) {
+  if constexpr (NP <= 2) {
+#pragma unroll
+    for (int i = 0; i < NP; ++i) c[i] = __ldg(p + i);
+  } else {
+#pragma unroll
+    for (int i = 0; i < NP; i += 4) {
+      const float4 t = __ldg(reinterpret_cast<const float4 *>(p + i));
+      c[i] = t.x;
+      if (i + 1 < NP) c[i + 1] = t.y;
+      if (i + 2 < NP) c[i + 2] = t.z;
+      if (i + 3 < NP) c[i + 3] = t.w;
+    }
+  }
+}
+
+// One block: `units` units of chunk ch.  A unit is a cell, assembled here, or one part of a split cell, whose sums
+// go to the scratch partials, summed in order by moments_combine.
 template <int NP>
 __device__ __forceinline__ void moments_fp32_body(const PlanView &v, const SweepArgs &a, const Layout &L, int ch,
-                                                  int64_t t0) {
-  extern __shared__ float coef[];   // [pair][3][NP] {w, w sin, w sin^2}, then [pair][2] {cos, sin}
-  float *csn = coef + 3 * NP * v.n_pairs;
-  for (int i = threadIdx.x; i < v.n_pairs * NP; i += blockDim.x) {
-    const int pr = i / NP, p = i - pr * NP;
-    const float w = v.polar[i].wf, sz = v.polar[i].sinzf;
-    coef[(pr * 3 + 0) * NP + p] = w;
-    coef[(pr * 3 + 1) * NP + p] = w * sz;
-    coef[(pr * 3 + 2) * NP + p] = (w * sz) * sz;
-  }
-  for (int i = threadIdx.x; i < v.n_pairs; i += blockDim.x) {
-    csn[2 * i] = v.pairs[i].cf;
-    csn[2 * i + 1] = v.pairs[i].sf;
-  }
-  __syncthreads();
+                                                  int64_t block, int units) {
+  extern __shared__ __align__(16) unsigned char msmem[];
+  constexpr int kStride = fold_stride(NP), kRow = fold_row(NP);
+  constexpr int kTogether = NP <= 4 ? kRunSegments : kRunSegments / 2;   // segments in flight together (registers)
   const int g0 = ch * L.gc;
   const int gcount = min(L.gc, v.G - g0);
-  const int64_t t = t0 + threadIdx.x;
-  if (ch == 0 && t == 0) const_cast<double *>(a.scale)[3] = 1.0;   // the state is in this step's scale now
-  if (t >= v.n_munits * gcount) return;
-  const int64_t unit = t / gcount;
-  const int gi = (int)(t - unit * gcount);
-  const int2 um = v.n_mmulti ? v.munit[unit] : make_int2((int)unit, 0);   // no split cell: unit = cell
-  const int cell = um.x;
-  const int g = g0 + gi;
-  const int4 *gent = v.gent + ch * v.gent_chunk;
+  const int64_t u0 = block * units;
+  if (u0 >= v.n_munits) return;
+  const int nu = (int)min((int64_t)units, v.n_munits - u0);
+  const int64_t r0 = v.unit_off[u0];
+  const int nr = (int)(v.unit_off[u0 + nu] - r0);
+  GatherRun *runs = reinterpret_cast<GatherRun *>(msmem);
+  float *P = reinterpret_cast<float *>(runs + nr);   // [3][run][group]
+  const int nt = nr * gcount;
+  {
+    const int4 *src = reinterpret_cast<const int4 *>(v.gent + ch * v.gent_chunk + r0);
+    for (int i = threadIdx.x; i < nr * (int)(sizeof(GatherRun) / 16); i += blockDim.x)
+      copy16_async(reinterpret_cast<int4 *>(runs) + i, src + i);
+    cp_async_commit();
+    cp_async_wait<0>();
+  }
+  __syncthreads();
+  if (ch == 0 && block == 0 && threadIdx.x == 0)
+    const_cast<double *>(a.scale)[3] = 1.0;   // the state is in this step's scale now
+  // 1. the runs' sums
   const float *I = (const float *)a.I;
-  float hi[kOutputs], lo[kOutputs];
+  {
+    int r = (int)threadIdx.x / gcount, gi = (int)threadIdx.x - r * gcount;
+    const int dr = (int)blockDim.x / gcount, dg = (int)blockDim.x - dr * gcount;
+    for (int t = threadIdx.x; t < nt; t += blockDim.x) {
+      const GatherRun &run = runs[r];
+      const int2 pc = *reinterpret_cast<const int2 *>(&run.pair);
+      float P0 = 0.f, P1 = 0.f, P2 = 0.f;
+      float c0[NP], c1[NP], c2[NP];
+      const float *cf = v.fold + pc.x * kStride;
+      load_fold<NP>(cf, c0);
+      load_fold<NP>(cf + kRow, c1);
+      load_fold<NP>(cf + 2 * kRow, c2);
 #pragma unroll
-  for (int k = 0; k < kOutputs; ++k) hi[k] = lo[k] = 0.f;
-  const int64_t ce0 = v.cell_off[cell], ce1 = v.cell_off[cell + 1];
-  const int64_t e0 = ce0 + (int64_t)um.y * kPartEntries;
-  const int ne = (int)min(ce1 - e0, (int64_t)kPartEntries);   // entries of this part (a multiple of kGatherBatch)
-  const bool split = ce1 - ce0 > kPartEntries;
-  const int4 *ep = gent + e0;
-  int cur = ne > 0 ? (__ldg(&ep->w) >> 1) : 0;
-  int run = 0;   // entries in the current FP32 partial sums
-  float P0 = 0.f, P1 = 0.f, P2 = 0.f;
-  auto flush = [&]() {
-    const float cf = csn[2 * cur], sf = csn[2 * cur + 1];
-    two_sum_add(hi[0], lo[0], P0);
-    two_sum_add(hi[1], lo[1], cf * P1);
-    two_sum_add(hi[2], lo[2], sf * P1);
-    two_sum_add(hi[3], lo[3], (cf * cf) * P2);
-    two_sum_add(hi[4], lo[4], (cf * sf) * P2);
-    two_sum_add(hi[5], lo[5], (sf * sf) * P2);
-  };
-  // up to 3 polar cosines the entries of the next batch are loaded while this batch's state loads are in flight;
-  // at 4 that costs the occupancy it buys (measured with the factors formed here), so each batch loads its own
-  constexpr bool kPrefetch = NP <= 3;
-  int4 en[kGatherBatch];
-  if (kPrefetch && ne > 0) {
+      for (int k0 = 0; k0 < kRunSegments; k0 += kTogether) {
+        float dv[kTogether][2][NP];
 #pragma unroll
-    for (int b = 0; b < kGatherBatch; ++b) en[b] = __ldg(ep + b);
-  }
-  for (int e = 0; e < ne; e += kGatherBatch) {
-    if constexpr (!kPrefetch) {
-      // the line holding the entries two batches ahead is fetched into L2 now (no registers held): the entry
-      // loads below then hit in cache instead of waiting on DRAM before the state loads that depend on them
-      if (e + 2 * kGatherBatch < ne)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(ep + e + 2 * kGatherBatch));
+        for (int k = 0; k < kTogether; ++k) {
+          const int4 s = run.seg[k0 + k];
+          load_dev_if<NP>(k0 + k < pc.y, I + gather_slot(s.x, s.z, gi) * NP, dv[k][0]);
+          load_dev_if<NP>(k0 + k < pc.y, I + gather_slot(s.y, s.w, gi) * NP, dv[k][1]);
+        }
 #pragma unroll
-      for (int b = 0; b < kGatherBatch; ++b) en[b] = __ldg(ep + e + b);
-    }
-    float dv[kGatherBatch][NP];
+        for (int k = 0; k < kTogether; ++k) {   // an absent segment adds zeros (its area and values)
+          const float af = run.area[k0 + k];
 #pragma unroll
-    for (int b = 0; b < kGatherBatch; ++b) load_dev_cg<NP>(I + gather_slot(en[b].x, en[b].y, gi) * NP, dv[b]);
-    int2 zw[kGatherBatch];
+          for (int sense = 0; sense < 2; ++sense) {
+            float S0 = 0.f, S1 = 0.f, S2 = 0.f;
 #pragma unroll
-    for (int b = 0; b < kGatherBatch; ++b) zw[b] = make_int2(en[b].z, en[b].w);
-    if (kPrefetch && e + kGatherBatch < ne) {
-#pragma unroll
-      for (int b = 0; b < kGatherBatch; ++b) en[b] = __ldg(ep + e + kGatherBatch + b);
-    }
-#pragma unroll
-    for (int b = 0; b < kGatherBatch; ++b) {
-      const int pr = zw[b].y >> 1;
-      if (pr != cur || run == kPairRun) {
-        flush();
-        cur = pr;
-        run = 0;
-        P0 = P1 = P2 = 0.f;
+            for (int p = 0; p < NP; ++p) {
+              S0 = fmaf(c0[p], dv[k][sense][p], S0);
+              S1 = fmaf(c1[p], dv[k][sense][p], S1);
+              S2 = fmaf(c2[p], dv[k][sense][p], S2);
+            }
+            P0 = fmaf(af, S0, P0);
+            P1 = fmaf(sense ? -af : af, S1, P1);
+            P2 = fmaf(af, S2, P2);
+          }
+        }
       }
-      ++run;
-      const float *c0 = coef + pr * 3 * NP;
-      float S0 = 0.f, S1 = 0.f, S2 = 0.f;
-#pragma unroll
-      for (int p = 0; p < NP; ++p) {
-        S0 = fmaf(c0[p], dv[b][p], S0);
-        S1 = fmaf(c0[NP + p], dv[b][p], S1);
-        S2 = fmaf(c0[2 * NP + p], dv[b][p], S2);
+      P[t] = P0;
+      P[nt + t] = P1;
+      P[2 * nt + t] = P2;
+      r += dr;
+      gi += dg;
+      if (gi >= gcount) {
+        gi -= gcount;
+        ++r;
       }
-      const float af = __int_as_float(zw[b].x);
-      P0 = fmaf(af, S0, P0);
-      P1 = fmaf((zw[b].y & 1) ? -af : af, S1, P1);
-      P2 = fmaf(af, S2, P2);
     }
   }
-  if (ne > 0) flush();
-  // FP64 work here is per (cell, group), not per update: conversions by integer operations, one add per sum
-  double D[kOutputs];
+  __syncthreads();
+  // 2. the units' sums
+  for (int k = threadIdx.x; k < nu * gcount; k += blockDim.x) {
+    const int ul = k / gcount, gi = k - ul * gcount;
+    const int64_t unit = u0 + ul;
+    const int2 um = v.n_mmulti ? v.munit[unit] : make_int2((int)unit, 1);
+    const int rb = (int)(v.unit_off[unit] - r0), re = (int)(v.unit_off[unit + 1] - r0);
+    f32x2 hi[3] = {0, 0, 0}, lo[3] = {0, 0, 0};   // (E, Fx), (Fy, Nxx), (Nxy, Nyy)
+#pragma unroll 4
+    for (int r = rb; r < re; ++r) {
+      const float2 cs = *reinterpret_cast<const float2 *>(&runs[r].cf);
+      const int t = r * gcount + gi;
+      const float P0 = P[t], P1 = P[nt + t], P2 = P[2 * nt + t];
+      two_sum_add2(hi[0], lo[0], pack2(P0, cs.x * P1));
+      two_sum_add2(hi[1], lo[1], mul2(pack2(cs.y, cs.x * cs.x), pack2(P1, P2)));
+      two_sum_add2(hi[2], lo[2], mul2(pack2(cs.x * cs.y, cs.y * cs.y), pack2(P2, P2)));
+    }
+    // FP64 work here is per (cell, group), not per update: conversions by integer operations, one add per sum
+    double D[kOutputs];
 #pragma unroll
-  for (int k = 0; k < kOutputs; ++k) D[k] = f32_to_f64(hi[k]) + f32_to_f64(lo[k]);
-  if (!split) {
-    assemble_cell(v, a, cell, g, D);
-  } else {
-    double *ps = v.mscratch + (((int64_t)ch * v.n_munits + unit) * kOutputs) * L.gc + gi;
+    for (int o = 0; o < 3; ++o) {
+      const float2 h = unpack2(hi[o]), l = unpack2(lo[o]);
+      D[2 * o] = f32_to_f64(h.x) + f32_to_f64(l.x);
+      D[2 * o + 1] = f32_to_f64(h.y) + f32_to_f64(l.y);
+    }
+    if (um.y == 1) {
+      assemble_cell(v, a, um.x, g0 + gi, D);
+    } else {
+      double *ps = v.mscratch + (((int64_t)ch * v.n_munits + unit) * kOutputs) * L.gc + gi;
 #pragma unroll
-    for (int k = 0; k < kOutputs; ++k) ps[k * L.gc] = D[k];
+      for (int o = 0; o < kOutputs; ++o) ps[o * L.gc] = D[o];
+    }
   }
 }
 
@@ -782,21 +866,19 @@ __global__ void __launch_bounds__(128) moments_combine_batch_kernel(const BatchI
   moments_combine_body(b.v, b.a, b.L, m.y, (int64_t)m.z * blockDim.x);
 }
 
-// blocks per SM: 7 up to 3 polar cosines (72 registers: the next batch's entries are loaded while the current
-// batch's state loads are in flight), 8 at 4, 5 beyond
+// 72 registers up to 4 polar cosines (64 spill: 3517 us a step at 512^2 x 17, 72 3437), 80 beyond
 template <int NP>
-__global__ void __launch_bounds__(128, NP <= 3 ? 7 : NP == 4 ? 8 : 5)
-    moments_fp32_kernel(PlanView v, SweepArgs a, Layout L) {
-  moments_fp32_body<NP>(v, a, L, blockIdx.y, (int64_t)blockIdx.x * blockDim.x);
+__global__ void __launch_bounds__(kMomentBlock, NP <= 4 ? 7 : 6) moments_fp32_kernel(PlanView v, SweepArgs a, Layout L) {
+  moments_fp32_body<NP>(v, a, L, blockIdx.y, blockIdx.x, v.munit_block[((int)blockIdx.y + 1) * L.gc > v.G]);
 }
 
-// Batched: block j handles threads 128 map[j].z .. of chunk map[j].y of instance map[j].x.
+// Batched: block j is block map[j].z, of map[j].w units a block, of chunk map[j].y of instance map[j].x.
 template <int NP>
-__global__ void __launch_bounds__(128, NP <= 3 ? 7 : NP == 4 ? 8 : 5)
+__global__ void __launch_bounds__(kMomentBlock, NP <= 4 ? 7 : 6)
     moments_fp32_batch_kernel(const BatchInst *inst, const int4 *map) {
   const int4 m = map[blockIdx.x];
   const BatchInst &b = inst[m.x];
-  moments_fp32_body<NP>(b.v, b.a, b.L, m.y, (int64_t)m.z * blockDim.x);
+  moments_fp32_body<NP>(b.v, b.a, b.L, m.y, m.z, m.w);
 }
 
 // f = N / (c E) per group (Eq. 7 with the cell averages of Eq. 15); <f>_E = sum_g N_g / (c sum_g E_g).
@@ -1153,11 +1235,10 @@ cudaError_t launch_sweep_fp32(const PlanView &v, const SweepArgs &a, cudaStream_
 
 cudaError_t launch_moments_fp32(const PlanView &v, const SweepArgs &a, cudaStream_t st) {
   const Layout L = layout_for(v, MOLC_FP32);
-  const int64_t blocks = (v.n_munits * L.gc + 127) / 128;
+  const int64_t blocks = moment_blocks(v, v.G >= L.gc * L.n_chunks ? v.munit_block[0] : std::min(v.munit_block[0], v.munit_block[1]));
   if (blocks > 0x7fffffff || L.n_chunks > 65535) return cudaErrorInvalidConfiguration;
   const dim3 grid((unsigned)blocks, (unsigned)L.n_chunks);
-  const size_t smem = (size_t)v.n_pairs * (3 * v.n_polar + 2) * sizeof(float);
-  if (smem > kMaxGatherSmem) return cudaErrorInvalidConfiguration;
+  const size_t smem = v.msmem;
   switch (v.n_polar) {
 #define MOLC_MOMENTS(NP)                                                                                       \
   case NP:                                                                                                     \
@@ -1166,7 +1247,7 @@ cudaError_t launch_moments_fp32(const PlanView &v, const SweepArgs &a, cudaStrea
                                            (int)smem);                                                         \
       if (e != cudaSuccess) return e;                                                                          \
     }                                                                                                          \
-    moments_fp32_kernel<NP><<<grid, 128, smem, st>>>(v, a, L);                                                 \
+    moments_fp32_kernel<NP><<<grid, kMomentBlock, smem, st>>>(v, a, L);                                                 \
     break;
     MOLC_MOMENTS(1)
     MOLC_MOMENTS(2)
@@ -1280,7 +1361,6 @@ cudaError_t launch_sweep_fp32_batch(const BatchInst *inst, const int2 *map, int 
 cudaError_t launch_moments_fp32_batch(const BatchInst *inst, const int4 *map, int blocks, int n_polar,
                                       size_t smem, cudaStream_t st) {
   if (blocks <= 0) return cudaSuccess;
-  if (smem > kMaxGatherSmem) return cudaErrorInvalidConfiguration;
   switch (n_polar) {
 #define MOLC_MOMENTS_B(NP)                                                                                     \
   case NP:                                                                                                     \
@@ -1289,7 +1369,7 @@ cudaError_t launch_moments_fp32_batch(const BatchInst *inst, const int4 *map, in
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);            \
       if (e != cudaSuccess) return e;                                                                          \
     }                                                                                                          \
-    moments_fp32_batch_kernel<NP><<<blocks, 128, smem, st>>>(inst, map);                                       \
+    moments_fp32_batch_kernel<NP><<<blocks, kMomentBlock, smem, st>>>(inst, map);                                       \
     break;
     MOLC_MOMENTS_B(1)
     MOLC_MOMENTS_B(2)
