@@ -87,7 +87,7 @@ __device__ __forceinline__ void ray_balance_max(unsigned long long *word, double
 
 
 // Eddington factors of one (cell, group) from the moments just assembled (Eq. 7 with the cell averages of
-// Eq. 15): f = N / (c E), 0 where E = 0.  The same operations as closure_cells, so molc_sweep_closure and
+// Eq. 15): f = N / (c E), 0 where E = 0.  The same operations as closure_kernel, so molc_sweep_closure and
 // molc_sweep + molc_closure give the same bits.
 __device__ __forceinline__ void eddington_factors(const SweepArgs &a, int64_t idx, double E, double nxx, double nxy,
                                                   double nyy) {
