@@ -158,6 +158,7 @@ __device__ __forceinline__ PolarFix load_polar(const PolarFix *p) {
 // Input checks, cell entries and cleared accumulators; one thread per (group, cell), cells fastest (an entry is one
 // 32-byte sector, the accumulators are cleared in memory order).
 __global__ void __launch_bounds__(256) prep_fp64_kernel(PlanView v, SweepArgs a) {
+  chain_next();
   const int64_t n = (int64_t)v.G * v.ncell, stride = (int64_t)gridDim.x * blockDim.x;
   bool bad = false;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -182,6 +183,7 @@ __global__ void __launch_bounds__(256) prep_fp64_kernel(PlanView v, SweepArgs a)
 constexpr int kFinalCells = 32, kFinalGroups = 8;
 __global__ void __launch_bounds__(kFinalCells *kFinalGroups) finalize_fp64_kernel(PlanView v, SweepArgs a) {
   __shared__ double sm[kOutputs][kFinalGroups][kFinalCells + 1];
+  chain_wait();
   const int c0 = blockIdx.x * kFinalCells, g0 = blockIdx.y * kFinalGroups;
   const int nc = min(kFinalCells, v.ncell - c0), ng = min(kFinalGroups, v.G - g0);
   for (int k = threadIdx.x; k < nc * kOutputs * kFinalGroups; k += blockDim.x) {
@@ -217,6 +219,7 @@ __global__ void __launch_bounds__(128, NPT >= 4 ? 3 : 4) sweep_fp64_kernel(PlanV
   constexpr bool FACES = EXTRA == kSweepFaces, BAL = EXTRA == kSweepBalance;
   static_assert(!BAL || NPT == 1, "the balance check follows one ray per thread");
   __shared__ u64 table[64];
+  chain_next();
   if (threadIdx.x < 64) table[threadIdx.x] = kExp2Table[threadIdx.x];
   __syncthreads();
   const int NP = v.n_polar, Q = v.G * NP;
@@ -236,6 +239,7 @@ __global__ void __launch_bounds__(128, NPT >= 4 ? 3 : 4) sweep_fp64_kernel(PlanV
   const int nseg = tr.nseg;
   const int64_t seg0 = sense ? tr.seg_off + nseg - 1 : tr.seg_off;
   const int sstep = sense ? -1 : 1;
+  chain_wait();
   const double Iin = a.bnd[(sense ? tr.entry_minus : tr.entry_plus) * v.G + g];
   const double inv_cdt = a.inv_cdt;
   const bool pairs2 = NPT % 2 == 0;   // 16-byte aligned: even rows, even offset
@@ -394,8 +398,7 @@ cudaError_t launch_fp64(const PlanView &v, const SweepArgs &a, cudaStream_t st) 
   const int n_chunks = v.n_polar / NPT;
   const int64_t blocks = (v.n_tracks * 2 * (int64_t)v.G * n_chunks + 127) / 128;
   if (blocks > 0x7fffffff) return cudaErrorInvalidConfiguration;
-  sweep_fp64_kernel<NPT, EXTRA><<<(unsigned)blocks, 128, 0, st>>>(v, a, n_chunks);
-  return cudaGetLastError();
+  return launch_chained(chained(v), sweep_fp64_kernel<NPT, EXTRA>, (unsigned)blocks, 128, 0, st, v, a, n_chunks);
 }
 
 }  // namespace
@@ -409,8 +412,7 @@ cudaError_t launch_prep_fp64(const PlanView &v, const SweepArgs &a, cudaStream_t
 cudaError_t launch_finalize_fp64(const PlanView &v, const SweepArgs &a, cudaStream_t st) {
   const dim3 grid((unsigned)((v.ncell + kFinalCells - 1) / kFinalCells),
                   (unsigned)((v.G + kFinalGroups - 1) / kFinalGroups));
-  finalize_fp64_kernel<<<grid, kFinalCells * kFinalGroups, 0, st>>>(v, a);
-  return cudaGetLastError();
+  return launch_chained(chained(v), finalize_fp64_kernel, grid, kFinalCells * kFinalGroups, 0, st, v, a);
 }
 
 cudaError_t launch_sweep_fp64(const PlanView &v, const SweepArgs &a, cudaStream_t st) {

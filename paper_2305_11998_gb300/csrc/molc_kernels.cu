@@ -102,13 +102,17 @@ __device__ __forceinline__ void prep_tiles(const PlanView &v, const SweepArgs &a
 }
 
 __global__ void __launch_bounds__(128) prep_kernel(PlanView v, SweepArgs a, Layout L) {
+  chain_next();
+  chain_wait();
   prep_tiles(v, a, L, blockIdx.y, blockIdx.x, gridDim.x, blockIdx.x == 0 && blockIdx.y == 0);
 }
 
 // Batched (FP32): block j prepares tile map[j].z of chunk map[j].y of instance map[j].x.
 __global__ void __launch_bounds__(128) prep_batch_kernel(const BatchInst *inst, const int4 *map) {
+  chain_next();
   const int4 m = map[blockIdx.x];
   const BatchInst &b = inst[m.x];
+  chain_wait();
   prep_tiles(b.v, b.a, b.L, m.y, m.z, 1 << 30, m.w != 0);
 }
 
@@ -405,15 +409,17 @@ __device__ __forceinline__ void sweep_fp32_body(const PlanView &v, const SweepAr
   const float fx = FACES ? (float)((sense ? -1.0 : 1.0) * v.pairs[tr.pair].c) : 0.f;
   const float fy = FACES ? (float)((sense ? -1.0 : 1.0) * v.pairs[tr.pair].s) : 0.f;
   const float width = FACES ? (float)tr.width : 0.f;
+  // records of steps 0..D-1; then everything the kernels before this one write
+  int2 recs[kSteps];
+#pragma unroll
+  for (int k = 0; k < kSteps; ++k) recs[k] = k < nseg ? ld_record(rec + k * rstep) : make_int2(0, 0);
+  chain_wait();
   // entering intensity (scaled), split like B so that I_in - B keeps the precision of the difference
   const double bin = live ? a.bnd[(sense ? tr.entry_minus : tr.entry_plus) * v.G + g] * a.scale[0] : 0.0;
   const float in_hi = (float)bin, in_lo = (float)(bin - (double)in_hi);
   const float rescale = (float)a.scale[3];   // power of two: the stored deviations to this step's scale
 
-  // prologue: records of steps 0..D-1; groups 0..D-2 = {deviations k, table k (k <= D-3)}
-  int2 recs[kSteps];
-#pragma unroll
-  for (int k = 0; k < kSteps; ++k) recs[k] = k < nseg ? ld_record(rec + k * rstep) : make_int2(0, 0);
+  // prologue: groups 0..D-2 = {deviations k, table k (k <= D-3)}
 #pragma unroll
   for (int k = 0; k < kSteps - 1; ++k) {
     if constexpr (COOP) {
@@ -580,6 +586,7 @@ __device__ __forceinline__ void sweep_fp32_body(const PlanView &v, const SweepAr
 template <int NP, int D, int EXTRA = kSweepPlain>
 __global__ void __launch_bounds__(kSweepBlock) sweep_fp32_kernel(PlanView v, SweepArgs a, Layout L) {
   __shared__ SweepSmem<NP, D> sm;
+  chain_next();
   sweep_fp32_body<NP, D, EXTRA>(v, a, L, v.block_order[blockIdx.x], sm);
 }
 
@@ -587,6 +594,7 @@ __global__ void __launch_bounds__(kSweepBlock) sweep_fp32_kernel(PlanView v, Swe
 template <int NP, int D>
 __global__ void __launch_bounds__(kSweepBlock) sweep_fp32_batch_kernel(const BatchInst *inst, const int2 *map) {
   __shared__ SweepSmem<NP, D> sm;
+  chain_next();
   const int2 m = map[blockIdx.x];
   const BatchInst &b = inst[m.x];
   sweep_fp32_body<NP, D>(b.v, b.a, b.L, m.y, sm);
@@ -728,6 +736,7 @@ template <int NP>
 __device__ __forceinline__ void moments_fp32_body(const PlanView &v, const SweepArgs &a, const Layout &L, int ch,
                                                   int64_t block, int units) {
   extern __shared__ __align__(16) unsigned char msmem[];
+  chain_next();
   constexpr int kStride = fold_stride(NP), kRow = fold_row(NP);
   constexpr int kTogether = NP <= 4 ? kRunSegments : kRunSegments / 2;   // segments in flight together (registers)
   const int g0 = ch * L.gc;
@@ -748,6 +757,7 @@ __device__ __forceinline__ void moments_fp32_body(const PlanView &v, const Sweep
     cp_async_wait<0>();
   }
   __syncthreads();
+  chain_wait();   // the runs are the plan's; the state is the sweep's
   if (ch == 0 && block == 0 && threadIdx.x == 0)
     const_cast<double *>(a.scale)[3] = 1.0;   // the state is in this step's scale now
   // 1. the runs' sums
@@ -857,12 +867,14 @@ __device__ __forceinline__ void moments_combine_body(const PlanView &v, const Sw
 }
 
 __global__ void __launch_bounds__(128) moments_combine_kernel(PlanView v, SweepArgs a, Layout L) {
+  chain_wait();
   moments_combine_body(v, a, L, blockIdx.y, (int64_t)blockIdx.x * blockDim.x);
 }
 
 __global__ void __launch_bounds__(128) moments_combine_batch_kernel(const BatchInst *inst, const int4 *map) {
   const int4 m = map[blockIdx.x];
   const BatchInst &b = inst[m.x];
+  chain_wait();
   moments_combine_body(b.v, b.a, b.L, m.y, (int64_t)m.z * blockDim.x);
 }
 
@@ -1122,6 +1134,7 @@ __device__ __forceinline__ void update_scale(unsigned long long mbits, double *h
 __global__ void __launch_bounds__(256) update_scale_kernel(const double *B, int64_t n, const double *bnd, int nb,
                                                          double *header) {
   __shared__ unsigned long long red[8];
+  chain_next();
   unsigned long long *mx = reinterpret_cast<unsigned long long *>(header + 2);
   unsigned int *cnt = reinterpret_cast<unsigned int *>(header + 4);
   unsigned long long m = 0;
@@ -1159,6 +1172,7 @@ __global__ void __launch_bounds__(256) update_scale_kernel(const double *B, int6
 template <class Inst>
 __global__ void __launch_bounds__(256) update_scale_map_kernel(const Inst *inst, const int4 *map) {
   __shared__ unsigned long long red[8];
+  chain_next();
   const int4 m = map[blockIdx.x];
   const Inst &b = inst[m.x];
   double *header = const_cast<double *>(b.a.scale);
@@ -1207,41 +1221,38 @@ cudaError_t launch_prep(const PlanView &v, const SweepArgs &a, cudaStream_t st) 
   if (L.gc > 32 || L.n_chunks > 65535) return cudaErrorInvalidConfiguration;
   const int n_tiles = (v.ncell + kPrepCells - 1) / kPrepCells;
   const dim3 grid((unsigned)std::min(n_tiles, 152 * 16), (unsigned)L.n_chunks);
-  prep_kernel<<<grid, 128, 0, st>>>(v, a, L);
-  return cudaGetLastError();
+  return launch_chained(chained(v), prep_kernel, grid, 128, 0, st, v, a, L);
 }
 
 template <int D>
 static cudaError_t sweep_fp32_depth(const PlanView &v, const SweepArgs &a, const Layout &L, dim3 grid,
                                     cudaStream_t st) {
   switch (v.n_polar) {
-    case 1: sweep_fp32_kernel<1, D><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
-    case 2: sweep_fp32_kernel<2, D><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
-    case 3: sweep_fp32_kernel<3, D><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
-    case 4: sweep_fp32_kernel<4, D><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
-    case 5: sweep_fp32_kernel<5, D><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
-    case 6: sweep_fp32_kernel<6, D><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
-    case 7: sweep_fp32_kernel<7, D><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
-    case 8: sweep_fp32_kernel<8, D><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
+    case 1: return launch_chained(chained(v), sweep_fp32_kernel<1, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 2: return launch_chained(chained(v), sweep_fp32_kernel<2, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 3: return launch_chained(chained(v), sweep_fp32_kernel<3, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 4: return launch_chained(chained(v), sweep_fp32_kernel<4, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 5: return launch_chained(chained(v), sweep_fp32_kernel<5, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 6: return launch_chained(chained(v), sweep_fp32_kernel<6, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 7: return launch_chained(chained(v), sweep_fp32_kernel<7, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 8: return launch_chained(chained(v), sweep_fp32_kernel<8, D>, grid, kSweepBlock, 0, st, v, a, L);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <int EXTRA>
 cudaError_t sweep_fp32_extra(const PlanView &v, const SweepArgs &a, const Layout &L, dim3 grid, cudaStream_t st) {
   switch (v.n_polar) {
-    case 1: sweep_fp32_kernel<1, 4, EXTRA><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
-    case 2: sweep_fp32_kernel<2, 4, EXTRA><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
-    case 3: sweep_fp32_kernel<3, 4, EXTRA><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
-    case 4: sweep_fp32_kernel<4, 4, EXTRA><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
-    case 5: sweep_fp32_kernel<5, 4, EXTRA><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
-    case 6: sweep_fp32_kernel<6, 4, EXTRA><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
-    case 7: sweep_fp32_kernel<7, 4, EXTRA><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
-    case 8: sweep_fp32_kernel<8, 4, EXTRA><<<grid, kSweepBlock, 0, st>>>(v, a, L); break;
+    case 1: return launch_chained(chained(v), sweep_fp32_kernel<1, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 2: return launch_chained(chained(v), sweep_fp32_kernel<2, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 3: return launch_chained(chained(v), sweep_fp32_kernel<3, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 4: return launch_chained(chained(v), sweep_fp32_kernel<4, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 5: return launch_chained(chained(v), sweep_fp32_kernel<5, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 6: return launch_chained(chained(v), sweep_fp32_kernel<6, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 7: return launch_chained(chained(v), sweep_fp32_kernel<7, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 8: return launch_chained(chained(v), sweep_fp32_kernel<8, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_sweep_fp32(const PlanView &v, const SweepArgs &a, cudaStream_t st) {
@@ -1265,15 +1276,12 @@ cudaError_t launch_moments_fp32(const PlanView &v, const SweepArgs &a, cudaStrea
   if (blocks > 0x7fffffff || L.n_chunks > 65535) return cudaErrorInvalidConfiguration;
   const dim3 grid((unsigned)blocks, (unsigned)L.n_chunks);
   const size_t smem = v.msmem;
+  cudaError_t e = cudaSuccess;
   switch (v.n_polar) {
-#define MOLC_MOMENTS(NP)                                                                                       \
-  case NP:                                                                                                     \
-    if (smem > 48 * 1024) {                                                                                    \
-      cudaError_t e = cudaFuncSetAttribute(moments_fp32_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                           (int)smem);                                                         \
-      if (e != cudaSuccess) return e;                                                                          \
-    }                                                                                                          \
-    moments_fp32_kernel<NP><<<grid, kMomentBlock, smem, st>>>(v, a, L);                                                 \
+#define MOLC_MOMENTS(NP)                                                                                          \
+  case NP:                                                                                                        \
+    if (smem > 48 * 1024) e = cudaFuncSetAttribute(moments_fp32_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+    if (e == cudaSuccess) e = launch_chained(chained(v), moments_fp32_kernel<NP>, grid, kMomentBlock, smem, st, v, a, L);  \
     break;
     MOLC_MOMENTS(1)
     MOLC_MOMENTS(2)
@@ -1286,11 +1294,9 @@ cudaError_t launch_moments_fp32(const PlanView &v, const SweepArgs &a, cudaStrea
 #undef MOLC_MOMENTS
     default: return cudaErrorInvalidValue;
   }
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || v.n_mmulti == 0) return e;
   const dim3 cgrid((unsigned)(((int64_t)v.n_mmulti * L.gc + 127) / 128), (unsigned)L.n_chunks);
-  moments_combine_kernel<<<cgrid, 128, 0, st>>>(v, a, L);
-  return cudaGetLastError();
+  return launch_chained(chained(v), moments_combine_kernel, cgrid, 128, 0, st, v, a, L);
 }
 
 // Face moments from the face sums: E_f = D is / (c |f|), F_f, N_f = sums is / |f|; is = 1/scale of the state
@@ -1374,25 +1380,23 @@ cudaError_t launch_update_scale_map(const BatchInst *inst, const TileInst *tinst
 
 cudaError_t launch_prep_batch(const BatchInst *inst, const int4 *map, int blocks, cudaStream_t st) {
   if (blocks <= 0) return cudaSuccess;
-  prep_batch_kernel<<<blocks, 128, 0, st>>>(inst, map);
-  return cudaGetLastError();
+  return launch_chained(false, prep_batch_kernel, blocks, 128, 0, st, inst, map);
 }
 
 template <int D>
 static cudaError_t sweep_fp32_batch_depth(const BatchInst *inst, const int2 *map, int blocks, int n_polar,
                                           cudaStream_t st) {
   switch (n_polar) {
-    case 1: sweep_fp32_batch_kernel<1, D><<<blocks, kSweepBlock, 0, st>>>(inst, map); break;
-    case 2: sweep_fp32_batch_kernel<2, D><<<blocks, kSweepBlock, 0, st>>>(inst, map); break;
-    case 3: sweep_fp32_batch_kernel<3, D><<<blocks, kSweepBlock, 0, st>>>(inst, map); break;
-    case 4: sweep_fp32_batch_kernel<4, D><<<blocks, kSweepBlock, 0, st>>>(inst, map); break;
-    case 5: sweep_fp32_batch_kernel<5, D><<<blocks, kSweepBlock, 0, st>>>(inst, map); break;
-    case 6: sweep_fp32_batch_kernel<6, D><<<blocks, kSweepBlock, 0, st>>>(inst, map); break;
-    case 7: sweep_fp32_batch_kernel<7, D><<<blocks, kSweepBlock, 0, st>>>(inst, map); break;
-    case 8: sweep_fp32_batch_kernel<8, D><<<blocks, kSweepBlock, 0, st>>>(inst, map); break;
+    case 1: return launch_chained(false, sweep_fp32_batch_kernel<1, D>, blocks, kSweepBlock, 0, st, inst, map);
+    case 2: return launch_chained(false, sweep_fp32_batch_kernel<2, D>, blocks, kSweepBlock, 0, st, inst, map);
+    case 3: return launch_chained(false, sweep_fp32_batch_kernel<3, D>, blocks, kSweepBlock, 0, st, inst, map);
+    case 4: return launch_chained(false, sweep_fp32_batch_kernel<4, D>, blocks, kSweepBlock, 0, st, inst, map);
+    case 5: return launch_chained(false, sweep_fp32_batch_kernel<5, D>, blocks, kSweepBlock, 0, st, inst, map);
+    case 6: return launch_chained(false, sweep_fp32_batch_kernel<6, D>, blocks, kSweepBlock, 0, st, inst, map);
+    case 7: return launch_chained(false, sweep_fp32_batch_kernel<7, D>, blocks, kSweepBlock, 0, st, inst, map);
+    case 8: return launch_chained(false, sweep_fp32_batch_kernel<8, D>, blocks, kSweepBlock, 0, st, inst, map);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_sweep_fp32_batch(const BatchInst *inst, const int2 *map, int blocks, int n_polar, int depth,
@@ -1409,15 +1413,12 @@ cudaError_t launch_sweep_fp32_batch(const BatchInst *inst, const int2 *map, int 
 cudaError_t launch_moments_fp32_batch(const BatchInst *inst, const int4 *map, int blocks, int n_polar,
                                       size_t smem, cudaStream_t st) {
   if (blocks <= 0) return cudaSuccess;
+  cudaError_t e = cudaSuccess;
   switch (n_polar) {
-#define MOLC_MOMENTS_B(NP)                                                                                     \
-  case NP:                                                                                                     \
-    if (smem > 48 * 1024) {                                                                                    \
-      cudaError_t e = cudaFuncSetAttribute(moments_fp32_batch_kernel<NP>,                                      \
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);            \
-      if (e != cudaSuccess) return e;                                                                          \
-    }                                                                                                          \
-    moments_fp32_batch_kernel<NP><<<blocks, kMomentBlock, smem, st>>>(inst, map);                                       \
+#define MOLC_MOMENTS_B(NP)                                                                                          \
+  case NP:                                                                                                        \
+    if (smem > 48 * 1024) e = cudaFuncSetAttribute(moments_fp32_batch_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+    if (e == cudaSuccess) e = launch_chained(false, moments_fp32_batch_kernel<NP>, blocks, kMomentBlock, smem, st, inst, map);  \
     break;
     MOLC_MOMENTS_B(1)
     MOLC_MOMENTS_B(2)
@@ -1430,13 +1431,12 @@ cudaError_t launch_moments_fp32_batch(const BatchInst *inst, const int4 *map, in
 #undef MOLC_MOMENTS_B
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_moments_combine_batch(const BatchInst *inst, const int4 *map, int blocks, cudaStream_t st) {
   if (blocks <= 0) return cudaSuccess;
-  moments_combine_batch_kernel<<<blocks, 128, 0, st>>>(inst, map);
-  return cudaGetLastError();
+  return launch_chained(false, moments_combine_batch_kernel, blocks, 128, 0, st, inst, map);
 }
 
 
