@@ -8,7 +8,7 @@
 // products and six atomics are shared by its polar cosines.  The attenuation (Eqs. 12-13), two transcendental
 // functions and two divisions an update when taken in FP64, is evaluated on the integer pipe in 64-bit fixed point.
 // 128^2 cells, 17 groups, 8 x 64 directions, h/2 (3.64e8 updates): 48.3 ms with FP64 exp, expm1, two divisions and six
-// atomics an update on one thread per polar cosine; 7.3 ms so, the FP64 pipe 85-90 % busy (issue slots 30 %).
+// atomics an update on one thread per polar cosine; 7.6 ms so, the FP64 pipe 85-90 % busy (issue slots 30 %).
 #include <cuda_runtime.h>
 
 #include <cstdint>

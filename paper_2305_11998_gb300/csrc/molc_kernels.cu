@@ -896,7 +896,9 @@ __global__ void __launch_bounds__(kMomentBlock, NP <= 4 ? 7 : 6)
 // Closure and grey coefficients.  A block takes kRowCells cells, kRowGroups groups at a time: its threads load a
 // (group, cell) each (cells fastest) and form what belongs to the group; the sums over groups are then taken from shared
 // memory by one thread per (sum, cell), group by group in order.  One thread per cell, looping over the groups, left
-// 64 blocks of such serial chains of loads at 128^2 x 17 groups: 22.5 us the closure, 24.3 us the coefficients.
+// 64 blocks of such serial chains of loads at 128^2 x 17 groups.  There the closure took 19.5 us back to back with its
+// inputs in L2, now 11.2, bound by the FP64 pipe (one division a group and cell); the coefficients 13.5, now 17.5, but in
+// a step, after the sweep, the step is faster with them so (496 -> 487-492 us): more loads are in flight at first touch.
 constexpr int kRowCells = 32, kRowGroups = 8;
 
 // f = N / (c E) per group (Eq. 7 with the cell averages of Eq. 15); <f>_E = sum_g N_g / (c sum_g E_g).
@@ -1302,7 +1304,8 @@ cudaError_t launch_moments_fp32(const PlanView &v, const SweepArgs &a, cudaStrea
 // Face moments from the face sums: E_f = D is / (c |f|), F_f, N_f = sums is / |f|; is = 1/scale of the state
 // (1 for FP64), |f| = hy on x-faces, hx on y-faces.  A block turns kFaceRows faces x up to kFaceGroups groups of
 // [face][6][gc] sums into [g][face] outputs through shared memory: reading them a (face, group) per thread, faces
-// fastest, every lane had lines of its own (128^2 x 17 groups: 27.5 us).  The two divisors are taken once a block.
+// fastest, every lane had lines of its own (128^2 x 17 groups, back to back: 25.5 us, now 15.9; the bytes alone are 7).
+// The two divisors are taken once a block.
 constexpr int kFaceRows = 16, kFaceGroups = 32;
 __global__ void __launch_bounds__(256) face_moments_kernel(PlanView v, Layout L, const double *scale, double c, double hx,
                                                            double hy, molc_moments out) {
