@@ -13,7 +13,9 @@ namespace molc {
 // dependent launch: a kernel calls chain_next at once, so that the next one's blocks are placed and load the plan's
 // constants meanwhile, and chain_wait (until every earlier kernel of the chain has finished and its writes are visible)
 // before they touch anything else.  The first kernel of a step is launched plainly: it starts after all earlier work of
-// the stream, so nothing reaches back past it.  16^2 x 4 groups: FP64 49.2 -> 43.1 us a step, FP32 26.6 -> 25.5.  Larger
+// the stream, so nothing reaches back past it.  What an earlier kernel of the chain writes is read by ordinary loads after
+// chain_wait, never through the read-only path (__ldg, ld.global.nc): that path takes its data to be constant while the
+// kernel runs, and the wait orders ordinary loads only.  16^2 x 4 groups: FP64 49.2 -> 43.1 us a step, FP32 26.6 -> 25.5.  Larger
 // steps lose by it (512^2 x 17 groups 3411 -> 3986 us, a batch of 16 3616 -> 4593): blocks that join an SM before the kernel
 // ahead has left it live with that kernel's split of shared memory and L1.
 inline bool chained(const PlanView &v) { return 2 * v.n_tracks * v.G <= 152 * kSweepBlock; }

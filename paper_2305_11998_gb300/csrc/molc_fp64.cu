@@ -258,8 +258,9 @@ __global__ void __launch_bounds__(128, NPT >= 4 ? 3 : 4) sweep_fp64_kernel(PlanV
   };
   auto load_cell = [&](int cell, Cell64 &c) {
     if (a.cell64) {
+      // plain loads: the prep kernel writes the table while this kernel may already be resident (chain_wait)
       const double2 *q = reinterpret_cast<const double2 *>(a.cell64 + (int64_t)cell * v.G + g);
-      const double2 x = __ldg(q), y = __ldg(q + 1);
+      const double2 x = q[0], y = q[1];
       c.kt = x.x;
       c.r = x.y;
       c.B = y.x;
