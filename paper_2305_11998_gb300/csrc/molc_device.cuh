@@ -9,16 +9,24 @@
 
 namespace molc {
 
-// In a step of fewer walks than the SMs take in one block each (chained), the kernels follow one another by programmatic
-// dependent launch: a kernel calls chain_next at once, so that the next one's blocks are placed and load the plan's
-// constants meanwhile, and chain_wait (until every earlier kernel of the chain has finished and its writes are visible)
-// before they touch anything else.  The first kernel of a step is launched plainly: it starts after all earlier work of
-// the stream, so nothing reaches back past it.  What an earlier kernel of the chain writes is read by ordinary loads after
-// chain_wait, never through the read-only path (__ldg, ld.global.nc): that path takes its data to be constant while the
-// kernel runs, and the wait orders ordinary loads only.  16^2 x 4 groups: FP64 49.2 -> 43.1 us a step, FP32 26.6 -> 25.5.  Larger
-// steps lose by it (512^2 x 17 groups 3411 -> 3986 us, a batch of 16 3616 -> 4593): blocks that join an SM before the kernel
-// ahead has left it live with that kernel's split of shared memory and L1.
-inline bool chained(const PlanView &v) { return 2 * v.n_tracks * v.G <= 152 * kSweepBlock; }
+// In a small step the kernels follow one another by programmatic dependent launch: a kernel calls chain_next at once, so
+// that the next one's blocks are placed and load the plan's constants meanwhile, and chain_wait (until every earlier kernel
+// of the chain has finished and its writes are visible) before they touch anything else.  The first kernel of a step is
+// launched plainly: it starts after all earlier work of the stream, so nothing reaches back past it.  What an earlier kernel
+// of the chain writes is read by ordinary loads after chain_wait, never through the read-only path (__ldg, ld.global.nc):
+// that path takes its data to be constant while the kernel runs, and the wait orders ordinary loads only.
+//
+// A step is chained where its walks need no more blocks than there are SMs and the kernel ahead of its sweep is small too,
+// link by link, from 240 shapes timed with each link on and off (times over those of plain launches):
+//  - FP32, input preparation and moment gather: up to 4 blocks of the preparation an SM (0.78 to 1.00; beyond, 0.97 to 1.02).
+//  - FP32, the sweep: it keeps the split of shared memory and L1 it finds on an SM for its whole, long run, and its blocks
+//    go where the preparation leaves room, so this link pays only behind a preparation of at most one block an SM, and of
+//    half of that where a sweep block has more shared memory than the preparation's (from 5 polar cosines).  With the
+//    links above: 0.75 to 0.99; at 128 blocks of the preparation 0.91 with 4 polar cosines but 1.09 with 5 (0.97 without
+//    this link), at 473 1.32 (0.96), at 1458 (216^2 cells, 1 group) 2.6.
+//  - FP64: up to 48 blocks of the preparation (0.87 to 1.03); at 106 1.08, at 418 1.27.
+// 16^2 x 4 groups: FP64 49.2 -> 43.1 us a step, FP32 26.6 -> 25.5.
+inline bool few_walks(const PlanView &v) { return 2 * v.n_tracks * v.G <= 152 * kSweepBlock; }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class... K, class... A>

@@ -11,6 +11,7 @@
 // atomics an update on one thread per polar cosine; 7.6 ms so, the FP64 pipe 85-90 % busy (issue slots 30 %).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "molc_device.cuh"
@@ -394,6 +395,12 @@ __global__ void __launch_bounds__(128, NPT >= 4 ? 3 : 4) sweep_fp64_kernel(PlanV
   }
 }
 
+// Blocks of the preparation; whether an FP64 step is chained.
+int prep_blocks_fp64(const PlanView &v) {
+  return (int)std::min<int64_t>(((int64_t)v.G * v.ncell + 255) / 256, 152 * 8);
+}
+bool chained(const PlanView &v) { return few_walks(v) && prep_blocks_fp64(v) <= 48; }
+
 template <int NPT, int EXTRA>
 cudaError_t launch_fp64(const PlanView &v, const SweepArgs &a, cudaStream_t st) {
   const int n_chunks = v.n_polar / NPT;
@@ -405,8 +412,7 @@ cudaError_t launch_fp64(const PlanView &v, const SweepArgs &a, cudaStream_t st) 
 }  // namespace
 
 cudaError_t launch_prep_fp64(const PlanView &v, const SweepArgs &a, cudaStream_t st) {
-  const int64_t blocks = ((int64_t)v.G * v.ncell + 255) / 256;
-  prep_fp64_kernel<<<(unsigned)(blocks < 152 * 8 ? blocks : 152 * 8), 256, 0, st>>>(v, a);
+  prep_fp64_kernel<<<(unsigned)prep_blocks_fp64(v), 256, 0, st>>>(v, a);
   return cudaGetLastError();
 }
 

@@ -109,10 +109,8 @@ __global__ void __launch_bounds__(128) prep_kernel(PlanView v, SweepArgs a, Layo
 
 // Batched (FP32): block j prepares tile map[j].z of chunk map[j].y of instance map[j].x.
 __global__ void __launch_bounds__(128) prep_batch_kernel(const BatchInst *inst, const int4 *map) {
-  chain_next();
   const int4 m = map[blockIdx.x];
   const BatchInst &b = inst[m.x];
-  chain_wait();
   prep_tiles(b.v, b.a, b.L, m.y, m.z, 1 << 30, m.w != 0);
 }
 
@@ -594,7 +592,6 @@ __global__ void __launch_bounds__(kSweepBlock) sweep_fp32_kernel(PlanView v, Swe
 template <int NP, int D>
 __global__ void __launch_bounds__(kSweepBlock) sweep_fp32_batch_kernel(const BatchInst *inst, const int2 *map) {
   __shared__ SweepSmem<NP, D> sm;
-  chain_next();
   const int2 m = map[blockIdx.x];
   const BatchInst &b = inst[m.x];
   sweep_fp32_body<NP, D>(b.v, b.a, b.L, m.y, sm);
@@ -874,7 +871,6 @@ __global__ void __launch_bounds__(128) moments_combine_kernel(PlanView v, SweepA
 __global__ void __launch_bounds__(128) moments_combine_batch_kernel(const BatchInst *inst, const int4 *map) {
   const int4 m = map[blockIdx.x];
   const BatchInst &b = inst[m.x];
-  chain_wait();
   moments_combine_body(b.v, b.a, b.L, m.y, (int64_t)m.z * blockDim.x);
 }
 
@@ -1174,7 +1170,6 @@ __global__ void __launch_bounds__(256) update_scale_kernel(const double *B, int6
 template <class Inst>
 __global__ void __launch_bounds__(256) update_scale_map_kernel(const Inst *inst, const int4 *map) {
   __shared__ unsigned long long red[8];
-  chain_next();
   const int4 m = map[blockIdx.x];
   const Inst &b = inst[m.x];
   double *header = const_cast<double *>(b.a.scale);
@@ -1218,11 +1213,19 @@ int grid_for(int64_t n, int block) {
 
 }  // namespace
 
+// Blocks of the preparation over one chunk; which links of an FP32 step are chained.
+static int prep_blocks(const PlanView &v) { return std::min((v.ncell + kPrepCells - 1) / kPrepCells, 152 * 16); }
+static bool chained(const PlanView &v) {
+  return few_walks(v) && (int64_t)prep_blocks(v) * layout_for(v, MOLC_FP32).n_chunks <= 152 * 4;
+}
+static bool sweep_chained(const PlanView &v) {
+  return few_walks(v) && (int64_t)prep_blocks(v) * layout_for(v, MOLC_FP32).n_chunks <= (v.n_polar <= 4 ? 152 : 76);
+}
+
 cudaError_t launch_prep(const PlanView &v, const SweepArgs &a, cudaStream_t st) {
   const Layout L = layout_for(v, MOLC_FP32);
   if (L.gc > 32 || L.n_chunks > 65535) return cudaErrorInvalidConfiguration;
-  const int n_tiles = (v.ncell + kPrepCells - 1) / kPrepCells;
-  const dim3 grid((unsigned)std::min(n_tiles, 152 * 16), (unsigned)L.n_chunks);
+  const dim3 grid((unsigned)prep_blocks(v), (unsigned)L.n_chunks);
   return launch_chained(chained(v), prep_kernel, grid, 128, 0, st, v, a, L);
 }
 
@@ -1230,14 +1233,14 @@ template <int D>
 static cudaError_t sweep_fp32_depth(const PlanView &v, const SweepArgs &a, const Layout &L, dim3 grid,
                                     cudaStream_t st) {
   switch (v.n_polar) {
-    case 1: return launch_chained(chained(v), sweep_fp32_kernel<1, D>, grid, kSweepBlock, 0, st, v, a, L);
-    case 2: return launch_chained(chained(v), sweep_fp32_kernel<2, D>, grid, kSweepBlock, 0, st, v, a, L);
-    case 3: return launch_chained(chained(v), sweep_fp32_kernel<3, D>, grid, kSweepBlock, 0, st, v, a, L);
-    case 4: return launch_chained(chained(v), sweep_fp32_kernel<4, D>, grid, kSweepBlock, 0, st, v, a, L);
-    case 5: return launch_chained(chained(v), sweep_fp32_kernel<5, D>, grid, kSweepBlock, 0, st, v, a, L);
-    case 6: return launch_chained(chained(v), sweep_fp32_kernel<6, D>, grid, kSweepBlock, 0, st, v, a, L);
-    case 7: return launch_chained(chained(v), sweep_fp32_kernel<7, D>, grid, kSweepBlock, 0, st, v, a, L);
-    case 8: return launch_chained(chained(v), sweep_fp32_kernel<8, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 1: return launch_chained(sweep_chained(v), sweep_fp32_kernel<1, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 2: return launch_chained(sweep_chained(v), sweep_fp32_kernel<2, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 3: return launch_chained(sweep_chained(v), sweep_fp32_kernel<3, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 4: return launch_chained(sweep_chained(v), sweep_fp32_kernel<4, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 5: return launch_chained(sweep_chained(v), sweep_fp32_kernel<5, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 6: return launch_chained(sweep_chained(v), sweep_fp32_kernel<6, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 7: return launch_chained(sweep_chained(v), sweep_fp32_kernel<7, D>, grid, kSweepBlock, 0, st, v, a, L);
+    case 8: return launch_chained(sweep_chained(v), sweep_fp32_kernel<8, D>, grid, kSweepBlock, 0, st, v, a, L);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -1245,14 +1248,14 @@ static cudaError_t sweep_fp32_depth(const PlanView &v, const SweepArgs &a, const
 template <int EXTRA>
 cudaError_t sweep_fp32_extra(const PlanView &v, const SweepArgs &a, const Layout &L, dim3 grid, cudaStream_t st) {
   switch (v.n_polar) {
-    case 1: return launch_chained(chained(v), sweep_fp32_kernel<1, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
-    case 2: return launch_chained(chained(v), sweep_fp32_kernel<2, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
-    case 3: return launch_chained(chained(v), sweep_fp32_kernel<3, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
-    case 4: return launch_chained(chained(v), sweep_fp32_kernel<4, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
-    case 5: return launch_chained(chained(v), sweep_fp32_kernel<5, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
-    case 6: return launch_chained(chained(v), sweep_fp32_kernel<6, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
-    case 7: return launch_chained(chained(v), sweep_fp32_kernel<7, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
-    case 8: return launch_chained(chained(v), sweep_fp32_kernel<8, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 1: return launch_chained(sweep_chained(v), sweep_fp32_kernel<1, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 2: return launch_chained(sweep_chained(v), sweep_fp32_kernel<2, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 3: return launch_chained(sweep_chained(v), sweep_fp32_kernel<3, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 4: return launch_chained(sweep_chained(v), sweep_fp32_kernel<4, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 5: return launch_chained(sweep_chained(v), sweep_fp32_kernel<5, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 6: return launch_chained(sweep_chained(v), sweep_fp32_kernel<6, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 7: return launch_chained(sweep_chained(v), sweep_fp32_kernel<7, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
+    case 8: return launch_chained(sweep_chained(v), sweep_fp32_kernel<8, 4, EXTRA>, grid, kSweepBlock, 0, st, v, a, L);
     default: return cudaErrorInvalidValue;
   }
 }
