@@ -709,15 +709,18 @@ std::string device_signature(int dev) {
   return buf;
 }
 
-// Units a block of the moment gather takes in a chunk of gcount groups (no more than leave `blocks` blocks), and its
-// shared memory.
-int moment_units(const std::vector<int64_t> &unit_off, int gcount, int64_t blocks, size_t &smem) {
+// Units a block of the moment gather takes in a chunk of gcount groups, and its shared memory: as many as leave `blocks`
+// blocks, or more where the runs of so few would leave the block's threads idle in its first phase, as far as
+// moment_smem_most allows.
+int moment_units(const std::vector<int64_t> &unit_off, int gcount, int np, int64_t blocks, size_t &smem) {
   const int64_t n = (int64_t)unit_off.size() - 1;
-  for (int units = (int)std::max<int64_t>(1, std::min<int64_t>(kMomentBlock / gcount, n / blocks));; --units) {
+  const int64_t sums = std::max<int64_t>(1, unit_off.back() * gcount);   // (run, group) sums of all units
+  const int64_t fill = std::min((kMomentSums * n + sums - 1) / sums, n / kMomentFewBlocks);
+  for (int units = (int)std::max<int64_t>(1, std::min<int64_t>(kMomentBlock / gcount, std::max(fill, n / blocks)));; --units) {
     int64_t most = 0;
     for (int64_t u = 0; u < n; u += units) most = std::max(most, unit_off[std::min(n, u + units)] - unit_off[u]);
     smem = moment_smem(most, gcount);
-    if (units == 1 || smem <= kMomentSmem) return units;
+    if (units == 1 || smem <= moment_smem_most(np, gcount)) return units;
   }
 }
 
@@ -1430,9 +1433,9 @@ molc_status molc_create(const molc_grid *grid, const molc_quadrature *quad, cons
     for (int last = 0; last < 2; ++last) {
       const int gcount = last && p->G % gc32 ? p->G % gc32 : gc32;
       size_t smem = 0;
-      v.munit_block[last] = moment_units(unit_off, gcount, kMomentBlocks, smem);
+      v.munit_block[last] = moment_units(unit_off, gcount, p->n_polar, kMomentBlocks, smem);
       v.msmem = std::max(v.msmem, smem);
-      p->batch_munit[last] = moment_units(unit_off, gcount, 1, smem);
+      p->batch_munit[last] = moment_units(unit_off, gcount, p->n_polar, 1, smem);
       p->batch_msmem = std::max(p->batch_msmem, smem);
     }
   v.mmulti = p->d_mmulti;

@@ -700,7 +700,27 @@ __device__ __forceinline__ void load_dev_if(bool on, const float *p, float (&v)[
       asm("{.reg .pred q;\n setp.ne.s32 q, %3, 0;\n @q ld.global.cg.v2.f32 {%0, %1}, [%2];}"
           : "+f"(v[i]), "+f"(v[i + 1])
           : "l"(p + i), "r"((int)on) : "memory");
-  } else {
+  } else if constexpr (NP >= 5) {
+    // an odd number of values starts on an 8-byte boundary or 4 bytes past one: loads of two, and one of the value left
+    // over in front or behind
+    const bool past = ((uintptr_t)p & 4) != 0;
+    float w[NP], one = 0.f;
+#pragma unroll
+    for (int i = 0; i + 1 < NP; i += 2) {
+      w[i] = w[i + 1] = 0.f;
+      asm("{.reg .pred q;\n setp.ne.s32 q, %3, 0;\n @q ld.global.cg.v2.f32 {%0, %1}, [%2];}"
+          : "+f"(w[i]), "+f"(w[i + 1])
+          : "l"(p + i + past), "r"((int)on) : "memory");
+    }
+    asm("{.reg .pred q;\n setp.ne.s32 q, %2, 0;\n @q ld.global.cg.f32 %0, [%1];}"
+        : "+f"(one)
+        : "l"(p + (past ? 0 : NP - 1)), "r"((int)on) : "memory");
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      const float before = i == 0 ? one : w[i - 1], here = i == NP - 1 ? one : w[i];
+      v[i] = past ? before : here;
+    }
+  } else {   // 1 or 3
 #pragma unroll
     for (int i = 0; i < NP; ++i)
       asm("{.reg .pred q;\n setp.ne.s32 q, %2, 0;\n @q ld.global.cg.f32 %0, [%1];}"
@@ -735,7 +755,7 @@ __device__ __forceinline__ void moments_fp32_body(const PlanView &v, const Sweep
   extern __shared__ __align__(16) unsigned char msmem[];
   chain_next();
   constexpr int kStride = fold_stride(NP), kRow = fold_row(NP);
-  constexpr int kTogether = NP <= 4 ? kRunSegments : kRunSegments / 2;   // segments in flight together (registers)
+  constexpr int kTogether = moment_together(NP);   // segments in flight together
   const int g0 = ch * L.gc;
   const int gcount = min(L.gc, v.G - g0);
   const int64_t u0 = block * units;
@@ -874,15 +894,15 @@ __global__ void __launch_bounds__(128) moments_combine_batch_kernel(const BatchI
   moments_combine_body(b.v, b.a, b.L, m.y, (int64_t)m.z * blockDim.x);
 }
 
-// 72 registers up to 4 polar cosines (64 spill: 3517 us a step at 512^2 x 17, 72 3437), 80 beyond
+// (4 polar cosines: 72 registers; 64 spill, 3517 us a step at 512^2 x 17, 72 3437)
 template <int NP>
-__global__ void __launch_bounds__(kMomentBlock, NP <= 4 ? 7 : 6) moments_fp32_kernel(PlanView v, SweepArgs a, Layout L) {
+__global__ void __launch_bounds__(kMomentBlock, moment_sm_blocks(NP)) moments_fp32_kernel(PlanView v, SweepArgs a, Layout L) {
   moments_fp32_body<NP>(v, a, L, blockIdx.y, blockIdx.x, v.munit_block[((int)blockIdx.y + 1) * L.gc > v.G]);
 }
 
 // Batched: block j is block map[j].z, of map[j].w units a block, of chunk map[j].y of instance map[j].x.
 template <int NP>
-__global__ void __launch_bounds__(kMomentBlock, NP <= 4 ? 7 : 6)
+__global__ void __launch_bounds__(kMomentBlock, moment_sm_blocks(NP))
     moments_fp32_batch_kernel(const BatchInst *inst, const int4 *map) {
   const int4 m = map[blockIdx.x];
   const BatchInst &b = inst[m.x];
