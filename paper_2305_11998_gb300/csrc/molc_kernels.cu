@@ -911,12 +911,11 @@ __global__ void __launch_bounds__(kMomentBlock, moment_sm_blocks(NP))
   moments_fp32_body<NP>(b.v, b.a, b.L, m.y, m.z, m.w);
 }
 
-// Closure and grey coefficients.  A block takes kRowCells cells, kRowGroups groups at a time: its threads load a
-// (group, cell) each (cells fastest) and form what belongs to the group; the sums over groups are then taken from shared
-// memory by one thread per (sum, cell), group by group in order.  One thread per cell, looping over the groups, left
-// 64 blocks of such serial chains of loads at 128^2 x 17 groups.  There the closure took 19.5 us back to back with its
-// inputs in L2, now 11.2, bound by the FP64 pipe (one division a group and cell); the coefficients 13.5, now 17.5, but in
-// a step, after the sweep, the step is faster with them so (496 -> 487-492 us): more loads are in flight at first touch.
+// Closure.  A block takes kRowCells cells, kRowGroups groups at a time: its threads load a (group, cell) each (cells
+// fastest) and form what belongs to the group; the sums over groups are then taken from shared memory by one thread per
+// (sum, cell), group by group in order.  One thread per cell, looping over the groups, left 64 blocks of serial chains of
+// loads at 128^2 x 17 groups: 19.5 us back to back with its inputs in L2, so 11.2, bound by the FP64 pipe (one division a
+// group and cell).
 constexpr int kRowCells = 32, kRowGroups = 8;
 
 // f = N / (c E) per group (Eq. 7 with the cell averages of Eq. 15); <f>_E = sum_g N_g / (c sum_g E_g).
@@ -957,53 +956,68 @@ __global__ void __launch_bounds__(kRowCells *kRowGroups) closure_kernel(PlanView
 
 // Grey-problem coefficients (Eqs. 8-9), all in FP64: <kappa>_E, <kappa>_B, the flux-weighted
 // K_R = diag(<kappa>_|Fx|, <kappa>_|Fy|) and eta = sum_g (kappa_g - K_R) F_g / sum_g E_g.
-__global__ void __launch_bounds__(kRowCells *kRowGroups) grey_kernel(PlanView v, molc_moments m, const double *kappa,
-                                                                     const double *B, double *out) {
-  __shared__ double sm[5][kRowGroups][kRowCells];   // kappa, E, B, Fx, Fy
-  const int cl = threadIdx.x % kRowCells, gl = threadIdx.x / kRowCells;
-  const int cell = blockIdx.x * kRowCells + cl;
-  const bool in = cell < v.ncell;
+// One thread per cell with the loads of kGreyGroups groups in flight, in blocks of one warp so that small grids reach all
+// SMs; the FP64 pipe bounds it (twelve operations a group and cell).  Back to back: 128^2 x 17 groups 11.8 us (13.4 with a
+// group's loads in flight, 17.5 as blocks of cells x groups through shared memory), 512^2 x 17 126 (125, 211), 512^2 x 1
+// 44 (44, 49), 64^2 x 17 11.2 (13.6, 7.1).  The results are written last: they may lie over an input.
+constexpr int kGreyBlock = 32, kGreyGroups = 4;
+__global__ void __launch_bounds__(kGreyBlock) grey_kernel(PlanView v, molc_moments m, const double *kappa, const double *B,
+                                                          double *out) {
+  const int cell = blockIdx.x * kGreyBlock + threadIdx.x;
+  if (cell >= v.ncell) return;
   const int64_t n = v.ncell;
-  // sums 2 x and 2 x + 1 of thread row gl: of E, B, |Fx|, |Fy| and of kappa times it
-  const int x = 1 + gl / 2;
-  double sum = 0.0;
-  for (int g0 = 0; g0 < v.G; g0 += kRowGroups) {
-    if (in && g0 + gl < v.G) {
-      const int64_t i = (int64_t)(g0 + gl) * n + cell;
-      sm[0][gl][cl] = kappa[i];
-      sm[1][gl][cl] = m.E[i];
-      sm[2][gl][cl] = B[i];
-      sm[3][gl][cl] = fabs(m.Fx[i]);
-      sm[4][gl][cl] = fabs(m.Fy[i]);
+  double se = 0, ske = 0, sb = 0, skb = 0, sfx = 0, skfx = 0, sfy = 0, skfy = 0;
+  for (int g0 = 0; g0 < v.G; g0 += kGreyGroups) {
+    double k[kGreyGroups], E[kGreyGroups], b[kGreyGroups], fx[kGreyGroups], fy[kGreyGroups];
+#pragma unroll
+    for (int j = 0; j < kGreyGroups; ++j) {
+      if (g0 + j >= v.G) break;
+      const int64_t i = (int64_t)(g0 + j) * n + cell;
+      k[j] = kappa[i];
+      E[j] = m.E[i];
+      b[j] = B[i];
+      fx[j] = fabs(m.Fx[i]);
+      fy[j] = fabs(m.Fy[i]);
     }
-    __syncthreads();
-    for (int k = 0; k < min(kRowGroups, v.G - g0); ++k)
-      sum = gl & 1 ? fma(sm[0][k][cl], sm[x][k][cl], sum) : sum + sm[x][k][cl];
-    __syncthreads();
-  }
-  sm[0][gl][cl] = sum;
-  __syncthreads();
-  double mean = 0.0;   // of rows 0 to 3: <kappa>_E, <kappa>_B, K_Rx, K_Ry
-  if (gl < 4) {
-    const double s = sm[0][2 * gl][cl];
-    mean = s > 0 ? sm[0][2 * gl + 1][cl] / s : 0.0;
-    if (in) out[gl * n + cell] = mean;
-  }
-  const double se = sm[0][0][cl];
-  double eta = 0.0;   // rows 2 and 3: sum_g (kappa_g - K_R) F_g
-  for (int g0 = 0; g0 < v.G; g0 += kRowGroups) {
-    __syncthreads();
-    if (in && g0 + gl < v.G) {
-      const int64_t i = (int64_t)(g0 + gl) * n + cell;
-      sm[0][gl][cl] = kappa[i];
-      sm[3][gl][cl] = m.Fx[i];
-      sm[4][gl][cl] = m.Fy[i];
+#pragma unroll
+    for (int j = 0; j < kGreyGroups; ++j) {
+      if (g0 + j >= v.G) break;
+      se += E[j];
+      ske = fma(k[j], E[j], ske);
+      sb += b[j];
+      skb = fma(k[j], b[j], skb);
+      sfx += fx[j];
+      skfx = fma(k[j], fx[j], skfx);
+      sfy += fy[j];
+      skfy = fma(k[j], fy[j], skfy);
     }
-    __syncthreads();
-    if (gl == 2 || gl == 3)
-      for (int k = 0; k < min(kRowGroups, v.G - g0); ++k) eta = fma(sm[0][k][cl] - mean, sm[gl + 1][k][cl], eta);
   }
-  if ((gl == 2 || gl == 3) && in) out[(gl + 2) * n + cell] = se > 0 ? eta / se : 0.0;
+  const double kE = se > 0 ? ske / se : 0.0, kB = sb > 0 ? skb / sb : 0.0;
+  const double kx = sfx > 0 ? skfx / sfx : 0.0, ky = sfy > 0 ? skfy / sfy : 0.0;
+  double ex = 0, ey = 0;
+  for (int g0 = 0; g0 < v.G; g0 += kGreyGroups) {
+    double k[kGreyGroups], fx[kGreyGroups], fy[kGreyGroups];
+#pragma unroll
+    for (int j = 0; j < kGreyGroups; ++j) {
+      if (g0 + j >= v.G) break;
+      const int64_t i = (int64_t)(g0 + j) * n + cell;
+      k[j] = kappa[i];
+      fx[j] = m.Fx[i];
+      fy[j] = m.Fy[i];
+    }
+#pragma unroll
+    for (int j = 0; j < kGreyGroups; ++j) {
+      if (g0 + j >= v.G) break;
+      ex = fma(k[j] - kx, fx[j], ex);
+      ey = fma(k[j] - ky, fy[j], ey);
+    }
+  }
+  out[cell] = kE;
+  out[n + cell] = kB;
+  out[2 * n + cell] = kx;
+  out[3 * n + cell] = ky;
+  out[4 * n + cell] = se > 0 ? ex / se : 0.0;
+  out[5 * n + cell] = se > 0 ? ey / se : 0.0;
 }
 
 // Canonical segment averages <-> deviation state, Ibar = B_ref(cell) + delta: one block per (track, sense).  The
@@ -1379,7 +1393,7 @@ cudaError_t launch_face_moments(const PlanView &v, molc_precision prec, const do
 
 cudaError_t launch_grey(const PlanView &v, const molc_moments &m, const double *kappa, const double *B,
                         double *out, cudaStream_t st) {
-  grey_kernel<<<(v.ncell + kRowCells - 1) / kRowCells, kRowCells * kRowGroups, 0, st>>>(v, m, kappa, B, out);
+  grey_kernel<<<(v.ncell + kGreyBlock - 1) / kGreyBlock, kGreyBlock, 0, st>>>(v, m, kappa, B, out);
   return cudaGetLastError();
 }
 
