@@ -915,7 +915,8 @@ __global__ void __launch_bounds__(kMomentBlock, moment_sm_blocks(NP))
 // fastest) and form what belongs to the group; the sums over groups are then taken from shared memory by one thread per
 // (sum, cell), group by group in order.  One thread per cell, looping over the groups, left 64 blocks of serial chains of
 // loads at 128^2 x 17 groups: 19.5 us back to back with its inputs in L2, so 11.2, bound by the FP64 pipe (one division a
-// group and cell).
+// group and cell).  With one or two groups most of such a block has nothing to load, and one thread per cell is faster:
+// 512^2 x 1 group 13.7 us for 21.5, 400^2 x 2 13.8 for 17.9 (one thread per cell at 5 groups 18.9 for 18.7).
 constexpr int kRowCells = 32, kRowGroups = 8;
 
 // f = N / (c E) per group (Eq. 7 with the cell averages of Eq. 15); <f>_E = sum_g N_g / (c sum_g E_g).
@@ -952,6 +953,34 @@ __global__ void __launch_bounds__(kRowCells *kRowGroups) closure_kernel(PlanView
   const double se = sm[0][0][cl];
   const double inv = se > 0 ? 1.0 / (c * se) : 0.0;
   fgrey[(gl - 1) * (int64_t)v.ncell + cell] = sum * inv;
+}
+
+constexpr int kFewGroups = 2, kFewBlock = 128;
+template <bool GREY>
+__global__ void __launch_bounds__(kFewBlock) closure_few_kernel(PlanView v, molc_moments m, double c, double *fxx, double *fxy,
+                                                                double *fyy, double *fgrey) {
+  const int cell = blockIdx.x * kFewBlock + threadIdx.x;
+  if (cell >= v.ncell) return;
+  double se = 0, sxx = 0, sxy = 0, syy = 0;
+  for (int g = 0; g < v.G; ++g) {
+    const int64_t i = (int64_t)g * v.ncell + cell;
+    const double E = m.E[i], nxx = m.Nxx[i], nxy = m.Nxy[i], nyy = m.Nyy[i];
+    const double inv = E > 0 ? 1.0 / (c * E) : 0.0;
+    fxx[i] = nxx * inv;
+    fxy[i] = nxy * inv;
+    fyy[i] = nyy * inv;
+    if constexpr (GREY) {
+      se += E;
+      sxx += nxx;
+      sxy += nxy;
+      syy += nyy;
+    }
+  }
+  if constexpr (!GREY) return;
+  const double inv = se > 0 ? 1.0 / (c * se) : 0.0;
+  fgrey[cell] = sxx * inv;
+  fgrey[v.ncell + cell] = sxy * inv;
+  fgrey[2 * (int64_t)v.ncell + cell] = syy * inv;
 }
 
 // Grey-problem coefficients (Eqs. 8-9), all in FP64: <kappa>_E, <kappa>_B, the flux-weighted
@@ -1399,7 +1428,13 @@ cudaError_t launch_grey(const PlanView &v, const molc_moments &m, const double *
 
 cudaError_t launch_closure(const PlanView &v, const molc_moments &m, double c, double *fxx, double *fxy,
                            double *fyy, double *f_grey, cudaStream_t st) {
-  closure_kernel<<<(v.ncell + kRowCells - 1) / kRowCells, kRowCells * kRowGroups, 0, st>>>(v, m, c, fxx, fxy, fyy, f_grey);
+  const unsigned few = (unsigned)((v.ncell + kFewBlock - 1) / kFewBlock);
+  if (v.G > kFewGroups)
+    closure_kernel<<<(v.ncell + kRowCells - 1) / kRowCells, kRowCells * kRowGroups, 0, st>>>(v, m, c, fxx, fxy, fyy, f_grey);
+  else if (f_grey)
+    closure_few_kernel<true><<<few, kFewBlock, 0, st>>>(v, m, c, fxx, fxy, fyy, f_grey);
+  else
+    closure_few_kernel<false><<<few, kFewBlock, 0, st>>>(v, m, c, fxx, fxy, fyy, f_grey);
   return cudaGetLastError();
 }
 
