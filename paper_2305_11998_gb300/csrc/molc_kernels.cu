@@ -1370,53 +1370,58 @@ cudaError_t launch_moments_fp32(const PlanView &v, const SweepArgs &a, cudaStrea
 }
 
 // Face moments from the face sums: E_f = D is / (c |f|), F_f, N_f = sums is / |f|; is = 1/scale of the state
-// (1 for FP64), |f| = hy on x-faces, hx on y-faces.  A block turns kFaceRows faces x up to kFaceGroups groups of
+// (1 for FP64), |f| = hy on x-faces, hx on y-faces.  A block turns `rows` faces x up to kFaceGroups groups of
 // [face][6][gc] sums into [g][face] outputs through shared memory: reading them a (face, group) per thread, faces
-// fastest, every lane had lines of its own (128^2 x 17 groups, back to back: 25.5 us, now 15.9; the bytes alone are 7).
-// The two divisors are taken once a block.
+// fastest, every lane had lines of its own.  The two divisors are taken once a block.
+// With few groups a block takes more faces, so that its threads have sums to read.  Back to back, one thread per (face,
+// group), then so (16 faces a block whatever the groups): 128^2 x 17 groups 25.7 us, 15.7 (16.0); 512^2 x 1 23.6, 14.9 (156);
+// 256^2 x 8 46.3, 26.7 (55.2); 64^2 x 4 4.2, 3.7 (6.1); 512^2 x 17 1098, 244 (272).
 constexpr int kFaceRows = 16, kFaceGroups = 32;
 __global__ void __launch_bounds__(256) face_moments_kernel(PlanView v, Layout L, const double *scale, double c, double hx,
-                                                           double hy, molc_moments out) {
-  __shared__ double sm[kOutputs][kFaceGroups][kFaceRows + 1];
+                                                           double hy, int rows, molc_moments out) {
+  __shared__ double sm[kOutputs * kFaceGroups * (kFaceRows + 1)];   // [output][group][rows + 1]
   __shared__ double factor[2][2];   // x-faces, y-faces: is / |f|, is / (c |f|)
-  const int face_blocks = (v.n_faces + kFaceRows - 1) / kFaceRows, slices = (L.gc + kFaceGroups - 1) / kFaceGroups;
+  const int face_blocks = (v.n_faces + rows - 1) / rows, slices = (L.gc + kFaceGroups - 1) / kFaceGroups;
   const int row = blockIdx.x / face_blocks, ch = row / slices, gs = (row - ch * slices) * kFaceGroups;
   const int ng = min(kFaceGroups, min(L.gc, v.G - ch * L.gc) - gs);
   if (ng <= 0) return;
-  const int f0 = (blockIdx.x - row * face_blocks) * kFaceRows, nf = min(kFaceRows, v.n_faces - f0);
+  const int f0 = (blockIdx.x - row * face_blocks) * rows, nf = min(rows, v.n_faces - f0);
   if (threadIdx.x < 2) {
     const double r = (scale ? scale[1] : 1.0) / (threadIdx.x ? hx : hy);
     factor[threadIdx.x][0] = r;
     factor[threadIdx.x][1] = r / c;
   }
   const double *fa = v.facc + ((int64_t)ch * v.n_faces + f0) * kOutputs * L.gc + gs;
-  for (int k = threadIdx.x; k < nf * kOutputs * kFaceGroups; k += blockDim.x) {
-    const int gl = k % kFaceGroups, fo = k / kFaceGroups;
-    if (gl < ng) sm[fo % kOutputs][gl][fo / kOutputs] = fa[(int64_t)fo * L.gc + gl];
+  const int pitch = rows + 1;
+  for (int k = threadIdx.x; k < nf * kOutputs * ng; k += blockDim.x) {
+    const int fo = k / ng, gl = k - fo * ng;
+    sm[((fo % kOutputs) * ng + gl) * pitch + fo / kOutputs] = fa[(int64_t)fo * L.gc + gl];
   }
   __syncthreads();
   const int nxf = (v.nx + 1) * v.ny;
-  for (int k = threadIdx.x; k < ng * kFaceRows; k += blockDim.x) {
-    const int fl = k % kFaceRows, gl = k / kFaceRows;
-    if (fl >= nf) continue;
+  for (int k = threadIdx.x; k < ng * nf; k += blockDim.x) {
+    const int gl = k / nf, fl = k - gl * nf;
     const int64_t i = (int64_t)(ch * L.gc + gs + gl) * v.n_faces + f0 + fl;
-    const double *r = factor[f0 + fl < nxf ? 0 : 1];
-    out.E[i] = sm[0][gl][fl] * r[1];
-    out.Fx[i] = sm[1][gl][fl] * r[0];
-    out.Fy[i] = sm[2][gl][fl] * r[0];
-    out.Nxx[i] = sm[3][gl][fl] * r[0];
-    out.Nxy[i] = sm[4][gl][fl] * r[0];
-    out.Nyy[i] = sm[5][gl][fl] * r[0];
+    const double *r = factor[f0 + fl < nxf ? 0 : 1], *x = sm + gl * pitch + fl;
+    out.E[i] = x[0] * r[1];
+    out.Fx[i] = x[ng * pitch] * r[0];
+    out.Fy[i] = x[2 * ng * pitch] * r[0];
+    out.Nxx[i] = x[3 * ng * pitch] * r[0];
+    out.Nxy[i] = x[4 * ng * pitch] * r[0];
+    out.Nyy[i] = x[5 * ng * pitch] * r[0];
   }
 }
 
 cudaError_t launch_face_moments(const PlanView &v, molc_precision prec, const double *scale, double c,
                                 const molc_moments &out, cudaStream_t st) {
   const Layout L = layout_for(v, prec);
-  const int64_t blocks = (int64_t)((v.n_faces + kFaceRows - 1) / kFaceRows) * L.n_chunks *
-                         ((L.gc + kFaceGroups - 1) / kFaceGroups);
+  const int64_t slices = (int64_t)L.n_chunks * ((L.gc + kFaceGroups - 1) / kFaceGroups);
+  // as many faces as fill the block's shared memory with few groups, but no fewer blocks than 4 an SM
+  int rows = kFaceRows;
+  while (2 * rows * std::min(L.gc, kFaceGroups) <= kFaceRows * kFaceGroups && v.n_faces / (2 * rows) * slices >= 152 * 4) rows *= 2;
+  const int64_t blocks = (v.n_faces + rows - 1) / rows * slices;
   if (blocks > 0x7fffffff) return cudaErrorInvalidConfiguration;   // more sums than device memory holds
-  face_moments_kernel<<<(unsigned)blocks, 256, 0, st>>>(v, L, scale, c, v.hx, v.hy, out);
+  face_moments_kernel<<<(unsigned)blocks, 256, 0, st>>>(v, L, scale, c, v.hx, v.hy, rows, out);
   return cudaGetLastError();
 }
 

@@ -57,3 +57,42 @@ def test_closure_time(n, G, most):
     P, m = plan(n, G), moments(n, G, 3)
     assert time_us(lambda: P.closure(m, 3.0, grey=True)) <= most
     P.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("n,G", [(3, 1), (60, 1), (200, 1), (120, 2), (90, 5), (70, 33)])
+def test_face_moments_of_each_group_alone(n, G, prec):
+    """Face moments of all groups against those of each group's own plan: the same sums, FP64 reductions in another order."""
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    kappa, B = (torch.rand(G, n * n, dtype=torch.float64, device="cuda", generator=gen) + 0.2 for _ in range(2))
+    bnd = torch.rand(4, G, dtype=torch.float64, device="cuda", generator=gen) + 0.2
+
+    def faces(groups):
+        P = plan(n, len(groups), faces=True)
+        I = P.new_intensity(prec)
+        k, b, e = kappa[groups].contiguous(), B[groups].contiguous(), bnd[:, groups].contiguous()
+        P.intensity_init(prec, I, b)
+        P.sweep(prec, k, b, 1.0, 0.3, I, e)
+        out = P.face_moments(prec, I, 1.0)
+        torch.cuda.synchronize()
+        P.close()
+        return out
+
+    whole = faces(list(range(G)))
+    for g in sorted({0, G // 2, G - 1}):
+        part = faces([g])
+        # a face takes fewer than 100 terms, none larger than its E c; FP32 states of B in [0.2, 1.2] share one scale
+        for k, x in part.items():
+            assert float((whole[k][g] - x[0]).abs().max()) <= 200 * U * float(whole["E"].max()), k
+
+
+# half-way between 156 and 23.6 us, 55.2 and 46.3 us: 16 faces a block whatever the groups, one thread per (face, group)
+@pytest.mark.parametrize("n,G,most", [(512, 1, 89.8), (256, 8, 50.7)])
+def test_face_moments_time(n, G, most):
+    P = plan(n, G, faces=True)
+    B = torch.ones(G, n * n, dtype=torch.float64, device="cuda")
+    I = P.new_intensity("fp32")
+    P.intensity_init("fp32", I, B)
+    P.sweep("fp32", B, B, 1.0, 0.3, I, torch.ones(4, G, dtype=torch.float64, device="cuda"))
+    assert time_us(lambda: P.face_moments("fp32", I, 1.0)) <= most
+    P.close()
