@@ -41,7 +41,9 @@ cudaError_t launch_chained(bool chain, void (*kernel)(K...), dim3 grid, dim3 blo
   cfg.stream = st;
   cfg.attrs = &attr;
   cfg.numAttrs = chain ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+  if (e != cudaSuccess) cudaGetLastError();   // reported here, not by the next launch
+  return e;
 }
 
 // Not (x >= 0 and finite), decided on the bits (integer pipe; the FP64 pipe is narrow): +0, -0 and the positive

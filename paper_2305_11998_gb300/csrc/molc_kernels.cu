@@ -1340,6 +1340,16 @@ cudaError_t launch_sweep_fp32(const PlanView &v, const SweepArgs &a, cudaStream_
   }
 }
 
+// A kernel's limit of dynamic shared memory is the whole process's: it is set to the most that any plan's gather takes, the
+// same by every thread, not to this plan's size, which another thread could lower before the launch.
+template <class K>
+static cudaError_t allow_moment_smem(K *kernel) {
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)moment_smem(kPartSegments, 32));
+  if (e != cudaSuccess) cudaGetLastError();   // reported here, not by the next launch
+  return e;
+}
+
 cudaError_t launch_moments_fp32(const PlanView &v, const SweepArgs &a, cudaStream_t st) {
   const Layout L = layout_for(v, MOLC_FP32);
   const int64_t blocks = moment_blocks(v, v.G >= L.gc * L.n_chunks ? v.munit_block[0] : std::min(v.munit_block[0], v.munit_block[1]));
@@ -1350,7 +1360,7 @@ cudaError_t launch_moments_fp32(const PlanView &v, const SweepArgs &a, cudaStrea
   switch (v.n_polar) {
 #define MOLC_MOMENTS(NP)                                                                                          \
   case NP:                                                                                                        \
-    if (smem > 48 * 1024) e = cudaFuncSetAttribute(moments_fp32_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+    if (smem > 48 * 1024) e = allow_moment_smem(moments_fp32_kernel<NP>);                                        \
     if (e == cudaSuccess) e = launch_chained(chained(v), moments_fp32_kernel<NP>, grid, kMomentBlock, smem, st, v, a, L);  \
     break;
     MOLC_MOMENTS(1)
@@ -1499,7 +1509,7 @@ cudaError_t launch_moments_fp32_batch(const BatchInst *inst, const int4 *map, in
   switch (n_polar) {
 #define MOLC_MOMENTS_B(NP)                                                                                          \
   case NP:                                                                                                        \
-    if (smem > 48 * 1024) e = cudaFuncSetAttribute(moments_fp32_batch_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+    if (smem > 48 * 1024) e = allow_moment_smem(moments_fp32_batch_kernel<NP>);                                     \
     if (e == cudaSuccess) e = launch_chained(false, moments_fp32_batch_kernel<NP>, blocks, kMomentBlock, smem, st, inst, map);  \
     break;
     MOLC_MOMENTS_B(1)
