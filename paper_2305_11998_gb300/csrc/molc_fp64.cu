@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(128, NPT >= 4 ? 3 : 4) sweep_fp64_kernel(PlanV
   chain_wait();
   const double Iin = a.bnd[(sense ? tr.entry_minus : tr.entry_plus) * v.G + g];
   const double inv_cdt = a.inv_cdt;
-  const bool pairs2 = NPT % 2 == 0;   // 16-byte aligned: even rows, even offset
+  const bool pairs2 = NPT % 2 == 0;   // 16-byte aligned: even rows, even offset (and the state: launch_sweep_fp64)
   auto load_state = [&](const double *p, double (&d)[NPT]) {
     if (pairs2) {
 #pragma unroll
@@ -433,7 +433,9 @@ cudaError_t launch_sweep_fp64(const PlanView &v, const SweepArgs &a, cudaStream_
   constexpr int64_t kEnough = 152 * 512;
   const int64_t walks = v.n_tracks * 2 * (int64_t)v.G;
   int npt = v.n_polar < 8 ? v.n_polar : 8;
-  while (npt > 1 && (v.n_polar % npt || walks * (v.n_polar / npt) < kEnough)) --npt;
+  // an even number is loaded in pairs: not from a state that starts 8 bytes past a 16-byte boundary
+  const bool pairs = ((uintptr_t)a.I & 15) == 0;
+  while (npt > 1 && (v.n_polar % npt || walks * (v.n_polar / npt) < kEnough || (npt % 2 == 0 && !pairs))) --npt;
   switch (npt) {
     case 8: return launch_fp64<8, kSweepPlain>(v, a, st);
     case 7: return launch_fp64<7, kSweepPlain>(v, a, st);
