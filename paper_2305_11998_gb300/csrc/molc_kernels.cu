@@ -984,11 +984,13 @@ __global__ void __launch_bounds__(kFewBlock) closure_few_kernel(PlanView v, molc
 }
 
 // Grey-problem coefficients (Eqs. 8-9), all in FP64: <kappa>_E, <kappa>_B, the flux-weighted
-// K_R = diag(<kappa>_|Fx|, <kappa>_|Fy|) and eta = sum_g (kappa_g - K_R) F_g / sum_g E_g.
+// K_R = diag(<kappa>_|Fx|, <kappa>_|Fy|) and eta = sum_g (kappa_g - K_R) F_g / sum_g E_g.  The results are written last: they
+// may lie over an input.
 // One thread per cell with the loads of kGreyGroups groups in flight, in blocks of one warp so that small grids reach all
-// SMs; the FP64 pipe bounds it (twelve operations a group and cell).  Back to back: 128^2 x 17 groups 11.8 us (13.4 with a
-// group's loads in flight, 17.5 as blocks of cells x groups through shared memory), 512^2 x 17 126 (125, 211), 512^2 x 1
-// 44 (44, 49), 64^2 x 17 11.2 (13.6, 7.1).  The results are written last: they may lie over an input.
+// SMs; the FP64 pipe bounds it (twelve operations a group and cell).  Where that leaves less than a warp an SM the groups
+// are shared out too (grey_small_kernel).  Back to back, one thread per cell, blocks of cells x groups: 64^2 x 17 groups
+// 11.2 and 7.1 us (13.6 with one group's loads in flight), 100^2 x 37 21.6 and 26.9, 128^2 x 17 11.8 and 17.5 (13.4),
+// 512^2 x 17 126 and 211 (125), 512^2 x 1 44 and 49 (44).
 constexpr int kGreyBlock = 32, kGreyGroups = 4;
 __global__ void __launch_bounds__(kGreyBlock) grey_kernel(PlanView v, molc_moments m, const double *kappa, const double *B,
                                                           double *out) {
@@ -1047,6 +1049,57 @@ __global__ void __launch_bounds__(kGreyBlock) grey_kernel(PlanView v, molc_momen
   out[3 * n + cell] = ky;
   out[4 * n + cell] = se > 0 ? ex / se : 0.0;
   out[5 * n + cell] = se > 0 ? ey / se : 0.0;
+}
+
+// The same with a (group, cell) loaded by a thread of its own, as in closure_kernel.
+__global__ void __launch_bounds__(kRowCells *kRowGroups) grey_small_kernel(PlanView v, molc_moments m, const double *kappa,
+                                                                           const double *B, double *out) {
+  __shared__ double sm[5][kRowGroups][kRowCells];   // kappa, E, B, Fx, Fy
+  const int cl = threadIdx.x % kRowCells, gl = threadIdx.x / kRowCells;
+  const int cell = blockIdx.x * kRowCells + cl;
+  const bool in = cell < v.ncell;
+  const int64_t n = v.ncell;
+  // sums 2 x and 2 x + 1 of thread row gl: of E, B, |Fx|, |Fy| and of kappa times it
+  const int x = 1 + gl / 2;
+  double sum = 0.0;
+  for (int g0 = 0; g0 < v.G; g0 += kRowGroups) {
+    if (in && g0 + gl < v.G) {
+      const int64_t i = (int64_t)(g0 + gl) * n + cell;
+      sm[0][gl][cl] = kappa[i];
+      sm[1][gl][cl] = m.E[i];
+      sm[2][gl][cl] = B[i];
+      sm[3][gl][cl] = fabs(m.Fx[i]);
+      sm[4][gl][cl] = fabs(m.Fy[i]);
+    }
+    __syncthreads();
+    for (int k = 0; k < min(kRowGroups, v.G - g0); ++k)
+      sum = gl & 1 ? fma(sm[0][k][cl], sm[x][k][cl], sum) : sum + sm[x][k][cl];
+    __syncthreads();
+  }
+  sm[0][gl][cl] = sum;
+  __syncthreads();
+  double mean = 0.0;   // of rows 0 to 3: <kappa>_E, <kappa>_B, K_Rx, K_Ry
+  if (gl < 4) {
+    const double s = sm[0][2 * gl][cl];
+    mean = s > 0 ? sm[0][2 * gl + 1][cl] / s : 0.0;
+  }
+  const double se = sm[0][0][cl];
+  double eta = 0.0;   // rows 2 and 3: sum_g (kappa_g - K_R) F_g
+  for (int g0 = 0; g0 < v.G; g0 += kRowGroups) {
+    __syncthreads();
+    if (in && g0 + gl < v.G) {
+      const int64_t i = (int64_t)(g0 + gl) * n + cell;
+      sm[0][gl][cl] = kappa[i];
+      sm[3][gl][cl] = m.Fx[i];
+      sm[4][gl][cl] = m.Fy[i];
+    }
+    __syncthreads();
+    if (gl == 2 || gl == 3)
+      for (int k = 0; k < min(kRowGroups, v.G - g0); ++k) eta = fma(sm[0][k][cl] - mean, sm[gl + 1][k][cl], eta);
+  }
+  if (!in || gl >= 4) return;
+  out[gl * n + cell] = mean;
+  if (gl >= 2) out[(gl + 2) * n + cell] = se > 0 ? eta / se : 0.0;
 }
 
 // Canonical segment averages <-> deviation state, Ibar = B_ref(cell) + delta: one block per (track, sense).  The
@@ -1437,7 +1490,10 @@ cudaError_t launch_face_moments(const PlanView &v, molc_precision prec, const do
 
 cudaError_t launch_grey(const PlanView &v, const molc_moments &m, const double *kappa, const double *B,
                         double *out, cudaStream_t st) {
-  grey_kernel<<<(v.ncell + kGreyBlock - 1) / kGreyBlock, kGreyBlock, 0, st>>>(v, m, kappa, B, out);
+  if (v.ncell <= 152 * kGreyBlock)
+    grey_small_kernel<<<(v.ncell + kRowCells - 1) / kRowCells, kRowCells * kRowGroups, 0, st>>>(v, m, kappa, B, out);
+  else
+    grey_kernel<<<(v.ncell + kGreyBlock - 1) / kGreyBlock, kGreyBlock, 0, st>>>(v, m, kappa, B, out);
   return cudaGetLastError();
 }
 

@@ -10,7 +10,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,G", [(9, 6), (16, 17), (45, 33)])
+@pytest.mark.parametrize("n,G", [(9, 6), (16, 17), (45, 33), (69, 9), (70, 6), (75, 17)])   # up to 69^2 cells shared out by groups too
 @pytest.mark.parametrize("over", ["kappa", "B", "E", "Fx", "Fy"])
 def test_output_over_an_input(n, G, over):
     import paper_2305_11998_gb300 as molc
