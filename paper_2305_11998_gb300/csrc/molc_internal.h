@@ -17,19 +17,22 @@ constexpr int kMomentBlock = 128;    // FP32 moments: threads of a block
 // the loads in flight, and with odd np, whose pieces take several loads, the lines between them; shared memory is taken
 // from that in steps, and past a step it slows down at once (256^2 x 17, 3 x 48, h/2 with 22 KB 495 us, 30 KB 1113).
 //  - blocks of an SM and segments of a thread in flight: short pieces want more threads, long ones fewer loads each.
-//    248^2 x 17, 1 x 48, h/4 582 -> 512; 256^2 x 17, 2 x 56, h/2 444 -> 389; 256^2 x 32, 2 x 32, h/2 454 -> 400.
-//  - shared memory of a block: 256^2 x 17, 3 x 48, h/2 494 -> 472, 243^2 x 8, 5 x 60, h/2 473 -> 387 and 128^2 x 17, 7 x 48, h/2
-//    386 -> 232 (these two with loads of two values); 256^2 x 8, 4 x 32, h/4 291 -> 270, where 1 and 17 groups want 22 KB.
-// 3 polar cosines and few groups keep a loss against one thread walking a cell's list: 256^2 x 8, 3 x 40, h/4 357 -> 370
-// (402 before), in a batch 365 -> 395 (438 before); wider loads, fewer loads in flight and more blocks were all slower there.
+//    248^2 x 17, 1 x 48, h/4 578 -> 511; 256^2 x 17, 2 x 56, h/2 445 -> 410; 256^2 x 32, 2 x 32, h/2 451 -> 424; 256^2 x 8, 2 x
+//    40, h/4 281 -> 260, in a batch 300 -> 278 (9 blocks and 17 KB: the first 389, but batches at h/4 up to 16 % slower).
+//  - shared memory of a block: 256^2 x 17, 3 x 48, h/2 490 -> 472, 243^2 x 8, 5 x 60, h/2 472 -> 386 and 128^2 x 17, 7 x 48, h/2
+//    382 -> 232 (these two with loads of two values); 256^2 x 8, 4 x 32, h/4 293 -> 274, where 1 and 17 groups want 22 KB;
+//    138^2 x 2, 2 x 64, h/8 316 us a step with 22 KB, 277 with 18.
+// 3 polar cosines and few groups keep a loss against one thread walking a cell's list: 256^2 x 8, 3 x 40, h/4 358 -> 369
+// (398 before), in a batch 367 -> 396 (434 before); wider loads, fewer loads in flight and more blocks were all slower there.
 // A block takes as many units as leave kMomentBlocks blocks (24 an SM: 64^2 x 17 groups 157 us a step with 8, 137 with 24),
 // but no fewer than give its first phase kMomentSums (run, group) sums while two blocks an SM are left: 79^2 x 11 groups,
-// 2 x 12, h/2 70 -> 62 us a step, 128^2 x 1, 4 x 32 94 -> 91, 48^2 x 4, 4 x 24 43 -> 37.  A single unit may take more
+// 2 x 12, h/2 74 -> 62 us a step, 128^2 x 1, 4 x 32 98 -> 92, 48^2 x 4, 4 x 24 43 -> 37.  A single unit may take more
 // shared memory: at most kPartSegments runs, 61 KB with 32 groups.
 constexpr int64_t kMomentBlocks = 152 * 24, kMomentFewBlocks = 152 * 2, kMomentSums = 3 * kMomentBlock;
-__host__ __device__ constexpr int moment_sm_blocks(int np) { return np <= 2 ? 9 : np <= 4 ? 7 : 6; }
+__host__ __device__ constexpr int moment_sm_blocks(int np) { return np == 1 ? 9 : np == 2 ? 8 : np <= 4 ? 7 : 6; }
 constexpr size_t moment_smem_most(int np, int gcount) {
-  return np <= 2 ? 17 * 1024 : np % 2 ? 17 * 1024 + 768 : np == 4 && gcount >= 8 && gcount < 16 ? 24 * 1024 : 22 * 1024;
+  return np % 2 || (np == 2 && gcount < 8) ? 17 * 1024 + 768
+                                           : np == 4 && gcount >= 8 && gcount < 16 ? 24 * 1024 : 22 * 1024;
 }
 constexpr int kRunSegments = 4;      // FP32 moments: segments of one azimuth pair summed in FP32 (GatherRun)
 __host__ __device__ constexpr int moment_together(int np) { return np == 1 || np == 4 ? kRunSegments : kRunSegments / 2; }
