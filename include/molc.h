@@ -206,7 +206,8 @@ molc_status molc_sweep(molc_plan *plan, molc_precision prec, const double *kappa
  * know all of it in advance, once they are running: an embedding whose device memory is fully handed to
  * another allocator, or a time-stepping loop run under a fixed memory budget.  Neither this call nor its
  * set-up calls cudaMalloc, cudaFree or any other allocating routine.
- *  - Limit: the workspace is 48 bytes per (cell, group) for MOLC_FP64 (the accumulators) and 20 bytes per
+ *  - Limit: the workspace is 48 bytes per (cell, group) for MOLC_FP64 (the accumulators; the sweep's cell entries, 32
+ *    bytes more, are tabulated where both fit and formed on the fly, more slowly, where not) and 20 bytes per
  *    (cell, group) for MOLC_FP32 (the cell tables; groups padded to the plan's group chunk); a MOLC_TILED plan
  *    needs about 220 bytes per (cell, group) plus (polar cosines + 2) x 4 bytes per (characteristic piece,
  *    group); each part is rounded up to 256 bytes.  A plan that needs more than 64 MiB (e.g. more than ~1.4M
@@ -216,8 +217,8 @@ molc_status molc_sweep(molc_plan *plan, molc_precision prec, const double *kappa
  *    address with cudaGetSymbolAddress, which also loads the library's kernels on that device if that has
  *    not happened yet; later calls reuse the cached address.  Make that first call before any stream
  *    capture.
- *  - The FP64 accumulators must start at zero; every FP64 call clears them itself (cudaMemsetAsync on
- *    `stream`) before its kernels run, so nothing needs to be zeroed by the caller.  The FP32 cell tables are
+ *  - The FP64 accumulators must start at zero; the first kernel of every FP64 call clears them, so nothing needs to be
+ *    zeroed by the caller.  The FP32 cell tables are
  *    fully rewritten by every call; a tiled FP32 call also clears its control words, work-item flags and
  *    arrival counts (a few KB) before its kernels run.
  *  - There is ONE array per device, shared by every plan and stream in the process: calls that can overlap in

@@ -8,7 +8,8 @@
 // products and six atomics are shared by its polar cosines.  The attenuation (Eqs. 12-13), two transcendental
 // functions and two divisions an update when taken in FP64, is evaluated on the integer pipe in 64-bit fixed point.
 // 128^2 cells, 17 groups, 8 x 64 directions, h/2 (3.64e8 updates): 48.3 ms with FP64 exp, expm1, two divisions and six
-// atomics an update on one thread per polar cosine; 7.6 ms so, the FP64 pipe 85-90 % busy (issue slots 30 %).
+// atomics an update on one thread per polar cosine; 7.7 ms so, of which about ten FP64
+// operations an update take 5.8 ms at the measured rate.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -428,7 +429,7 @@ cudaError_t launch_sweep_fp64(const PlanView &v, const SweepArgs &a, cudaStream_
   // Polar cosines one thread carries: the largest divisor of their number, up to 8, that leaves 16 warps an SM
   // (152 x 512 threads).  More of them share a segment's products and atomics, but with fewer threads the short
   // characteristics end early and the long ones run on alone: 17 groups, 8 polar cosines, 128^2 cells (355k walks)
-  // 13.1 ms with 1, 9.4 with 2, 8.0 with 4, 7.3 with 8; 7 groups, 3 polar cosines, 75 x 52 cells (23k walks) 250 us
+  // 13.1 ms with 1, 9.4 with 2, 8.0 with 4, 7.7 with 8; 7 groups, 3 polar cosines, 75 x 52 cells (23k walks) 250 us
   // with 1 and 317 with 3; 7 groups, 4 polar cosines, 150 x 100 cells (45k walks) 838 us with 1, 743 with 2, 930 with 4.
   constexpr int64_t kEnough = 152 * 512;
   const int64_t walks = v.n_tracks * 2 * (int64_t)v.G;

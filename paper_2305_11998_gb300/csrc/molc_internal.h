@@ -37,7 +37,8 @@ constexpr size_t moment_smem_most(int np, int gcount) {
 constexpr int kRunSegments = 4;      // FP32 moments: segments of one azimuth pair summed in FP32 (GatherRun)
 __host__ __device__ constexpr int moment_together(int np) { return np == 1 || np == 4 ? kRunSegments : kRunSegments / 2; }
 constexpr int kSweepBlock = 128;     // FP32 sweep: work items (threads) per block = width of a state bundle
-constexpr size_t kMaxGatherSmem = 200 * 1024;  // FP32: the per-pair coefficients a plan may have, in bytes
+constexpr size_t kMaxGatherSmem = 200 * 1024;  // per-pair coefficients a plan may have, in bytes: what plans are refused beyond
+                                               // (the gather once held them in shared memory)
 
 // Device status bits (the first one set wins in molc_device_status).
 constexpr int kStatusNonfinite = 1;
@@ -246,7 +247,8 @@ cudaError_t launch_set_scale(const PlanView &v, molc_precision prec, const doubl
                              cudaStream_t st);
 // Batched FP32 kernels: one launch each over the blocks of all instances listed in a block map
 // (prep: int4 {instance, chunk, tile, check boundary}; sweep: int2 {instance, bundle}, one launch per
-// (polar count, staging depth) class; moments: int4 {instance, chunk, block, 0}, one launch per polar count;
+// (polar count, staging depth) class; moments: int4 {instance, chunk, block, units a block}, one launch per polar
+// count and amount of shared memory;
 // closure: int2 {instance, cell block}).
 // Sweep-time scale update of an FP32 state from max(B, boundary) (see update_scale in molc_kernels.cu).
 cudaError_t launch_update_scale(const PlanView &v, const double *B, const double *bnd, double *header,

@@ -613,10 +613,9 @@ __global__ void __launch_bounds__(kSweepBlock) sweep_fp32_batch_kernel(const Bat
 // a thread, depend on nothing but words already in shared memory, the runs of a cell are spread over the block, and the
 // second phase adds in step.  The FP32 sums run over the same terms in the same order as one thread's walk (run by run,
 // segment by segment, + sense before - sense), so the moments do not depend on how cells and runs are shared out.
-// A step, before and after (the gather alone is what changed): 512^2 x 17 groups, 4 polar cosines, h/2 3523 -> 3414 us;
-// 128^2 x 17, 8 polar cosines x 64, h/8 3035 -> 2818; 64^2 x 17, 4, h/4 154 -> 137; 160 x 120 x 17, 3, h/3 391 -> 367,
-// 1 polar cosine 128^2 x 17, h/2 186 -> 172; 6 polar cosines 427 -> 428; 40^2 paper layout at 1e-3 cm 2191 -> 2091;
-// 16^2 x 4 groups 34.5 -> 28; a batch of 16 problems of 32^2 to 256^2 3709 -> 3593.
+// A step with one thread walking a cell's list, then so (the gather alone is what changed): 512^2 x 17 groups, 4 polar
+// cosines, h/2 3523 -> 3430 us; 128^2 x 17, 8 polar cosines x 64, h/8 3035 -> 2812; 64^2 x 17, 4, h/4 154 -> 137; 40^2 paper
+// layout at 1e-3 cm 2191 -> 2081; 16^2 x 4 groups 34.5 -> 28; a batch of 16 problems of 32^2 to 256^2 3709 -> 3520.
 __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float x) {
   const float s = __fadd_rn(hi, x);
   const float bp = __fsub_rn(s, hi);
@@ -1107,8 +1106,8 @@ __global__ void __launch_bounds__(kRowCells *kRowGroups) grey_small_kernel(PlanV
 // take consecutive (step, group) pairs and, for each, the NP adjacent deviations of the state (a block reads runs of
 // groups x NP values and writes NP contiguous streams).  One thread per state row, looping over polar cosines and
 // groups, had every lane on rows of its own: 64^2 x 17 groups, 4 x 32 directions, h/4 (4.6e7 values, 0.55 GB)
-// 565 us either way; so it is 135 us out and 159 us in.  That is bound by the FP64 pipe (one addition a value, busy
-// 71 and 60 %; the power-of-two scalings and the conversions are integer operations), with DRAM at 3.5 TB/s next.
+// 565 us either way; so it is 135 us out and 159 us in.  That is bound by the FP64 pipe (one addition a value; the
+// power-of-two scalings and the conversions are integer operations), with DRAM at 3.5 TB/s next.
 // One thread's elements of a walk, (step, group) by (step, group): f(step, group).
 template <class F>
 __device__ __forceinline__ void for_walk(int nseg, int g_count, F f) {
@@ -1641,8 +1640,7 @@ cudaError_t launch_set_scale(const PlanView &v, molc_precision prec, const doubl
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// FP64 FMA throughput of this GPU (the bound of the plain FP64 sweep, which spends its time in FP64 exp/expm1
-// and FP64 atomics): every thread runs kFmaChains independent chains of kFmaIters dependent FMAs, so the FP64
+// FP64 FMA throughput of this GPU (the bound of the plain FP64 sweep, whose intensity updates and polar folds are FP64): every thread runs kFmaChains independent chains of kFmaIters dependent FMAs, so the FP64
 // pipe, not latency, limits the rate.  The chains' sum is compared with a value it never takes and stored, if it
 // did, to a static device variable, so that the work cannot be dropped and no pointer is needed.
 // ---------------------------------------------------------------------------------------------------------
